@@ -107,10 +107,24 @@ struct DensifyArgs {
     int64_t n_old, capacity, P;
 };
 
+constexpr uint32_t kDensifySplit = 4;
+
+// A block's new Gaussians are consecutive rows of every parameter array, so
+// the block first lists them (mean, log-scale, pixel) in shared memory and then
+// writes each array's span flat, consecutive threads consecutive floats.
+// kDensifySplit blocks share a chunk's rows (a frame has few chunks).
+// Bound: HBM writes (44 + 12 (deg + 1)^2 bytes a Gaussian).  One thread per
+// Gaussian writing its own rows, as before, stored 4 bytes of a 192-byte row at
+// a time: 38.0 us for 116k new SH3 Gaussians of a 640x480 frame, now 12.6 us
+// (57 us with one block a chunk and a division and a load in the SH loop).
 __global__ void __launch_bounds__(kSelThreads) densify_write_kernel(DensifyArgs a, ViewTable vt, const uint32_t *offsets)
 {
     __shared__ uint32_t tmp[kSelThreads / 32];
-    const int64_t first = (int64_t)blockIdx.x * kSelChunk + (int64_t)threadIdx.x * kSelItems;
+    __shared__ float s_mean[3 * kSelChunk];
+    __shared__ float s_ls[kSelChunk];
+    __shared__ uint16_t s_pix[kSelChunk];  // pixel of the row, from the chunk's first
+    const int64_t chunk0 = (int64_t)blockIdx.x * kSelChunk;
+    const int64_t first = chunk0 + (int64_t)threadIdx.x * kSelItems;
     bool sel[kSelItems];
     uint32_t c = 0;
     #pragma unroll
@@ -120,13 +134,17 @@ __global__ void __launch_bounds__(kSelThreads) densify_write_kernel(DensifyArgs 
         c += sel[k];
     }
     uint32_t total;
-    uint32_t off = offsets[blockIdx.x] + block_scan_u32(c, tmp, &total);
-    #pragma unroll 1
-    for (int k = 0; k < kSelItems; k++) {
-        if (!sel[k]) continue;
-        const int64_t p = first + k;
-        const int64_t g = a.n_old + off++;
-        if (g >= a.capacity) continue;
+    uint32_t row = block_scan_u32(c, tmp, &total);
+    #pragma unroll
+    for (int k = 0; k < kSelItems; k++)
+        if (sel[k]) s_pix[row++] = (uint16_t)(threadIdx.x * kSelItems + k);
+    __syncthreads();
+    const int64_t g0 = a.n_old + offsets[blockIdx.x];
+    // rows past the capacity are dropped; of the others this block writes [r0, r1)
+    const uint32_t m = g0 >= a.capacity ? 0u : (uint32_t)(a.capacity - g0 < total ? a.capacity - g0 : total);
+    const uint32_t r0 = m * blockIdx.y / kDensifySplit, r1 = m * (blockIdx.y + 1) / kDensifySplit;
+    for (uint32_t r = r0 + threadIdx.x; r < r1; r += kSelThreads) {
+        const int64_t p = chunk0 + s_pix[r];
         int v = 0;
         for (int w = 1; w < vt.n_views; w++)
             if (p >= vt.v[w].pix_base) v = w;
@@ -138,21 +156,33 @@ __global__ void __launch_bounds__(kSelThreads) densify_write_kernel(DensifyArgs 
         const float xc = (px - V.cx) / V.fx * d, yc = (py - V.cy) / V.fy * d, zc = d;
         const float *E = a.viewmats + 12 * v;
         const float qx = xc - E[3], qy = yc - E[7], qz = zc - E[11];
-        a.means[3 * g + 0] = E[0] * qx + E[4] * qy + E[8] * qz;
-        a.means[3 * g + 1] = E[1] * qx + E[5] * qy + E[9] * qz;
-        a.means[3 * g + 2] = E[2] * qx + E[6] * qy + E[10] * qz;
-        const float ls = logf(d / V.fx);  // one pixel on the image plane: r = d / f
-        a.log_scales[3 * g + 0] = ls;
-        a.log_scales[3 * g + 1] = ls;
-        a.log_scales[3 * g + 2] = ls;
-        a.quats[4 * g + 0] = 1.0f;
-        a.quats[4 * g + 1] = 0.0f;
-        a.quats[4 * g + 2] = 0.0f;
-        a.quats[4 * g + 3] = 0.0f;
-        a.opac[g] = a.opacity_logit;
-        float *shg = a.sh + (int64_t)a.sh_floats * g;
-        for (int k = 0; k < a.sh_floats; k++) shg[k] = 0.0f;
-        for (int ch = 0; ch < 3; ch++) shg[ch] = (a.rgb[3 * p + ch] - 0.5f) / kShC0;
+        s_mean[3 * r + 0] = E[0] * qx + E[4] * qy + E[8] * qz;
+        s_mean[3 * r + 1] = E[1] * qx + E[5] * qy + E[9] * qz;
+        s_mean[3 * r + 2] = E[2] * qx + E[6] * qy + E[10] * qz;
+        s_ls[r] = logf(d / V.fx);  // one pixel on the image plane: r = d / f
+    }
+    __syncthreads();
+    for (uint32_t e = 3 * r0 + threadIdx.x; e < 3 * r1; e += kSelThreads) {
+        a.means[3 * g0 + e] = s_mean[e];
+        a.log_scales[3 * g0 + e] = s_ls[e / 3];
+    }
+    for (uint32_t e = 4 * r0 + threadIdx.x; e < 4 * r1; e += kSelThreads) a.quats[4 * g0 + e] = (e & 3u) ? 0.0f : 1.0f;
+    for (uint32_t e = r0 + threadIdx.x; e < r1; e += kSelThreads) a.opac[g0 + e] = a.opacity_logit;
+    const uint32_t w = (uint32_t)a.sh_floats;
+    float *sh = a.sh + (int64_t)w * g0;
+    #pragma unroll 4
+    for (uint32_t e = 3 * r0 + threadIdx.x; e < 3 * r1; e += kSelThreads) {
+        const uint32_t r = e / 3, ch = e - 3 * r;
+        sh[(size_t)w * r + ch] = (a.rgb[3 * (chunk0 + s_pix[r]) + ch] - 0.5f) / kShC0;
+    }
+    // the higher bands: the span without each row's first three floats
+    const uint32_t dc = kSelThreads % w;
+    uint32_t col = threadIdx.x % w;
+    #pragma unroll 4
+    for (uint32_t e = w * r0 + threadIdx.x; e < w * r1; e += kSelThreads) {
+        if (col >= 3) sh[e] = 0.0f;
+        col += dc;
+        if (col >= w) col -= w;
     }
 }
 
@@ -185,21 +215,65 @@ struct RowArrays {
     int32_t count;
     const float *src[GS_MAX_COMPACT_ARRAYS];
     float *dst[GS_MAX_COMPACT_ARRAYS];
-    int32_t width[GS_MAX_COMPACT_ARRAYS];
+    uint32_t units[GS_MAX_COMPACT_ARRAYS];  // 16-byte (vec) or 4-byte units of a row
+    uint32_t rows[GS_MAX_COMPACT_ARRAYS];   // rows a block copies
+    uint32_t block0[GS_MAX_COMPACT_ARRAYS]; // the array's first block
+    bool vec[GS_MAX_COMPACT_ARRAYS];
 };
 
-// One thread per (row, array); copies kept rows to their new index.
-__global__ void compact_rows_kernel(const int32_t *__restrict__ new_index, int64_t n, RowArrays A)
+constexpr int kRowThreads = 256;
+constexpr int kRowUnroll = 8;
+constexpr int kRowUnits = kRowThreads * kRowUnroll;  // units a block copies (at least one row)
+
+// Kept rows of one array, from row0 on, as a flat span of units: consecutive
+// threads copy consecutive units, kRowUnroll of them in flight a thread.
+template <typename U>
+__device__ __forceinline__ void copy_rows(const int32_t *__restrict__ new_index, const U *__restrict__ src,
+                                          U *__restrict__ dst, int64_t row0, uint32_t rows, uint32_t units)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int a = blockIdx.y;
-    if (i >= n || a >= A.count) return;
-    const int32_t j = new_index[i];
-    if (j < 0) return;
-    const int w = A.width[a];
-    const float *s = A.src[a] + (int64_t)w * i;
-    float *d = A.dst[a] + (int64_t)w * j;
-    for (int k = 0; k < w; k++) d[k] = s[k];
+    const uint64_t span = (uint64_t)rows * units;
+    for (uint64_t e0 = threadIdx.x; e0 < span; e0 += kRowUnits) {
+        int64_t to[kRowUnroll];
+        U v[kRowUnroll];
+        #pragma unroll
+        for (int k = 0; k < kRowUnroll; k++) {
+            const uint64_t e = e0 + (uint64_t)k * kRowThreads;
+            to[k] = -1;
+            if (e < span) {
+                // a block's span is below 2^32 units unless a single row is larger
+                const uint32_t r = rows == 1 ? 0u : (uint32_t)e / units;
+                const int32_t j = new_index[row0 + r];
+                if (j >= 0) to[k] = (int64_t)units * j + (int64_t)(e - (uint64_t)r * units);
+            }
+        }
+        #pragma unroll
+        for (int k = 0; k < kRowUnroll; k++)
+            if (to[k] >= 0) v[k] = src[(int64_t)units * row0 + (int64_t)(e0 + (uint64_t)k * kRowThreads)];
+        #pragma unroll
+        for (int k = 0; k < kRowUnroll; k++)
+            if (to[k] >= 0) dst[to[k]] = v[k];
+    }
+}
+
+// Bound: HBM (every kept row read and written once, 4 bytes of index a row
+// and array).  A block copies a span of about 2,048 units of one array; rows
+// of a multiple of four floats move 16 bytes at a time.  A thread per row,
+// copying its row float by float, touched a 32-byte sector per 4-byte access:
+// 1,327 us for 15 arrays (SH3 parameters, m, v) of 1M rows, now 284 us
+// (1.42 GB, 5.0 TB/s).
+__global__ void __launch_bounds__(kRowThreads) compact_rows_kernel(const int32_t *__restrict__ new_index, int64_t n,
+                                                                   RowArrays A)
+{
+    int a = 0;
+    for (int k = 1; k < A.count; k++)
+        if (blockIdx.x >= A.block0[k]) a = k;
+    const int64_t row0 = (int64_t)(blockIdx.x - A.block0[a]) * A.rows[a];
+    const uint32_t rows = (uint32_t)(n - row0 < A.rows[a] ? n - row0 : A.rows[a]);
+    if (A.vec[a])
+        copy_rows(new_index, reinterpret_cast<const float4 *>(A.src[a]), reinterpret_cast<float4 *>(A.dst[a]), row0,
+                  rows, A.units[a]);
+    else
+        copy_rows(new_index, A.src[a], A.dst[a], row0, rows, A.units[a]);
 }
 
 }  // namespace gs
@@ -252,7 +326,7 @@ extern "C" gs_status_t gs_densify(const float *alpha, const float *target_rgb, c
     a.n_old = n_old;
     a.capacity = capacity;
     a.P = P;
-    densify_write_kernel<<<(unsigned)nb, kSelThreads, 0, s>>>(a, vt, counts);
+    densify_write_kernel<<<dim3((unsigned)nb, kDensifySplit), kSelThreads, 0, s>>>(a, vt, counts);
     return launch_status();
 }
 
@@ -280,18 +354,23 @@ extern "C" gs_status_t gs_compact_rows(const int32_t *new_index, int64_t n, cons
                                        int32_t n_arrays, void *stream)
 {
     if (!new_index || !arrays || n < 0 || n_arrays < 1 || n_arrays > GS_MAX_COMPACT_ARRAYS) return GS_ERR_INVALID_ARG;
-    RowArrays A;
+    RowArrays A = {};
     A.count = n_arrays;
-    for (int k = 0; k < GS_MAX_COMPACT_ARRAYS; k++) {
-        A.src[k] = k < n_arrays ? arrays[k].src : nullptr;
-        A.dst[k] = k < n_arrays ? arrays[k].dst : nullptr;
-        A.width[k] = k < n_arrays ? arrays[k].row_floats : 0;
-        if (k < n_arrays && (!A.src[k] || !A.dst[k] || A.width[k] < 1 || A.src[k] == A.dst[k]))
-            return GS_ERR_INVALID_ARG;
+    int64_t blocks = 0;
+    for (int k = 0; k < n_arrays; k++) {
+        const int32_t w = arrays[k].row_floats;
+        A.src[k] = arrays[k].src;
+        A.dst[k] = arrays[k].dst;
+        if (!A.src[k] || !A.dst[k] || w < 1 || A.src[k] == A.dst[k]) return GS_ERR_INVALID_ARG;
+        A.vec[k] = w % 4 == 0 && ((reinterpret_cast<uintptr_t>(A.src[k]) | reinterpret_cast<uintptr_t>(A.dst[k])) & 15) == 0;
+        A.units[k] = (uint32_t)(A.vec[k] ? w / 4 : w);
+        A.rows[k] = A.units[k] < (uint32_t)kRowUnits ? (uint32_t)kRowUnits / A.units[k] : 1u;
+        A.block0[k] = (uint32_t)blocks;
+        blocks += (n + A.rows[k] - 1) / A.rows[k];
+        if (blocks > 0x7fffffffLL) return GS_ERR_INVALID_ARG;
     }
     if (n == 0) return GS_OK;
-    dim3 grid((unsigned)((n + 255) / 256), (unsigned)n_arrays);
-    compact_rows_kernel<<<grid, 256, 0, as_stream(stream)>>>(new_index, n, A);
+    compact_rows_kernel<<<(unsigned)blocks, kRowThreads, 0, as_stream(stream)>>>(new_index, n, A);
     return launch_status();
 }
 
