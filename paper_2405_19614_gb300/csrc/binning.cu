@@ -4,8 +4,9 @@
 //
 // The result is the list a stable sort of the 64-bit keys (global tile << 32)
 // | bits(depth), values = Gaussian index, would give: per tile, entries by
-// depth, equal depths in index order.  It is built in two small sorts instead
-// of one wide one:
+// depth, equal depths in index order.  Unless the map crowds few tiles,
+// tile_lists.cu builds it tile by tile; here it is built in two small sorts
+// instead of one wide one:
 //   1. the drawn (view, Gaussian) records are compacted and sorted by depth
 //      (four 8-bit passes over 32-bit keys; ties stay in record order);
 //   2. every record emits one (tile id, depth rank) pair per tile it touches,
@@ -462,6 +463,14 @@ extern "C" gs_status_t gs_bin_sort(const gs_projected_t *proj, int64_t n, const 
     const int tile_passes = (bits_for(vt.n_tiles_total - 1) + 7) / 8 > 0 ? (bits_for(vt.n_tiles_total - 1) + 7) / 8 : 1;
     if (tile_passes > kMaxTilePasses) return GS_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
+    if (total > 0 && tile_lists_fit(total, vt.n_tiles_total)) {
+        if (!proj->rec || !proj->rect || !proj->tiles_touched || !proj->tile_mask) return GS_ERR_INVALID_ARG;
+        // the pair buffer holds the 64-bit words, a look-back region the list of
+        // long tiles' chunks, the record buffers (rz to recs, one after the
+        // other) the counting blocks' table
+        const size_t table_bytes = (size_t)(reinterpret_cast<char *>(w.lb[0]) - reinterpret_cast<char *>(w.rz[0]));
+        return tile_lists(proj, total, n, vt, bins, {w.small, w.lb[0], w.pk, w.rz[0], table_bytes}, s);
+    }
     if (cudaMemsetAsync(bins->ranges, 0, sizeof(uint32_t) * 2 * (size_t)vt.n_tiles_total, s) != cudaSuccess)
         return GS_ERR_CUDA;
     if (total == 0) {

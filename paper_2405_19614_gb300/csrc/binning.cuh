@@ -63,4 +63,16 @@ constexpr BinOffsets bin_offsets(int64_t n_records, int64_t cap)
     return o;
 }
 
+// The path of tile_lists.cu (tiles counted, scattered and sorted one by one)
+// and whether the sizes are for it.  buffers: small, >= 32 bytes; chunks, >= 8
+// bytes per 1024 pairs of capacity; words, 8 bytes per pair of capacity; table,
+// any size (a small one limits the blocks that count).
+struct TileListBuffers {
+    void *small, *chunks, *words, *table;
+    size_t table_bytes;
+};
+bool tile_lists_fit(int64_t n_records, int64_t n_tiles);
+gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, const ViewTable &vt, gs_bins_t *bins,
+                       const TileListBuffers &buf, cudaStream_t s);
+
 }  // namespace gs

@@ -1,0 +1,664 @@
+// a2 - a4 for maps that are not crowded into a few tiles: the tile lists by
+// counting, scattering and sorting each tile on its own.
+//
+//   1. tile_count_kernel adds up each tile's pairs and tile_scan_kernel turns
+//      the counts into every tile's [start, end) and lists the long tiles;
+//   2. tile_scatter_kernel writes each pair's (depth bits, Gaussian index) as
+//      one 64-bit word at its tile's next free slot (an atomic again, so the
+//      order within a tile is arbitrary here);
+//   3. tile_sort_kernel sorts each tile's words: depth first, equal depths by
+//      index.  The words of a tile are distinct, so the sorted list does not
+//      depend on the order they arrived in: it is the list a stable sort of
+//      the 64-bit keys (tile << 32) | depth bits gives;
+//   4. tile_merge_kernel puts together the chunks of the tiles of more than
+//      kTileChunk words (a rank by binary search in the other chunks); it has
+//      nothing to do on most calls.
+//
+// Against sorting all records by depth, emitting their pairs in that order and
+// sorting the pairs by tile id (binning.cu: 13 to 16 dependent launches, of
+// which a small map fills few blocks) this is five launches, reads each drawn
+// record twice and each pair twice, and has no pass over all pairs that waits
+// on its predecessors.  Bound: with many pairs the instruction issue of the
+// sort (about log^2 of the list length a word); on small maps the five
+// launches.  Kernel times, this against binning.cu:
+//   100k Gaussians, 640x480, 49k pairs            36 against 125 us
+//   300k Gaussians, 1200x680, 174k pairs          42 against 111 us
+//   1M, 8 views of 1200x680 (32x16 tiles), 4.0M   235 against 305 us
+//   4M, 16 views (lists up to 59,000), 28.2M      1.67 against 2.36 ms
+#include "binning.cuh"
+#include "common.cuh"
+
+namespace gs {
+
+constexpr int kListThreads = 256;
+constexpr int kSortGroup = 128;                    // threads that sort a tile
+constexpr int kSortBlock = 4 * kSortGroup;         // threads of a block: four tiles, or a long tile's chunk
+constexpr int kMergeThreads = 256;
+constexpr int kScanThreads = 1024;
+constexpr int kBlocksPerSm = 6;                    // counting and scattering blocks, resident
+constexpr size_t kMaxTileSmem = 64 * 1024;         // a view's tiles in shared memory (16,384)
+constexpr uint32_t kGroupWords = 16 * kSortGroup;  // words a group sorts (16 KB of shared memory)
+constexpr uint32_t kTileChunk = 16 * kSortBlock;   // words a block sorts (64 KB)
+
+// Words of the small region this path uses.
+struct ListState {
+    uint32_t n_long;     // chunks listed in long_chunks
+    uint32_t cut;        // 1: the pairs exceed the capacity and only the nearest are kept
+    uint32_t cut_z, cut_r;  // (depth bits, record id) of the last record kept
+    uint32_t cut_pairs;  // how many of its pairs
+};
+
+struct ListArgs {
+    const float *rec;
+    const uint2 *rect;
+    const unsigned long long *mask;
+    const uint32_t *tt;
+    uint32_t total, n;  // records (views x Gaussians), Gaussians
+    uint32_t cap;
+    uint2 *ranges;
+    uint32_t *n_pairs, *status;
+    ListState *state;
+    uint2 *long_chunks;         // (tile, chunk of kTileChunk) of the tiles longer than kGroupWords
+    unsigned long long *words;  // [cap] unsorted (depth bits, index)
+    uint32_t *table;  // [blocks][table_pitch] a block's first slot in each tile of its view
+    uint32_t table_pitch;
+    uint64_t *keys;
+    uint32_t *vals;
+};
+
+// A drawn record's tiles.
+struct Splat {
+    uint32_t tile0;        // tile of the rectangle's corner, within the view
+    uint32_t wh;           // width | height << 16
+    uint32_t z, idx;       // depth bits, Gaussian
+    uint32_t rbase;        // record 0 of the view
+    unsigned long long mask;
+};
+
+// The ordinal of a record's tile i (row-major in its rectangle) among its pairs.
+__device__ __forceinline__ uint32_t pair_ordinal(const Splat &s, uint32_t i)
+{
+    if ((s.wh & 0xffffu) * (s.wh >> 16) > 64) return i;
+    return (uint32_t)__popcll(s.mask & ((1ull << i) - 1ull));
+}
+
+// Whether a pair is among the nearest that fit (state.cut).
+__device__ __forceinline__ bool pair_kept(const ListState &st, const Splat &s, uint32_t i)
+{
+    if (s.z != st.cut_z) return s.z < st.cut_z;
+    if (s.rbase + s.idx != st.cut_r) return s.rbase + s.idx < st.cut_r;
+    return pair_ordinal(s, i) < st.cut_pairs;
+}
+
+// What a walk does with tile i of splat s, tile `tile` of the view.
+struct CountPut {
+    uint32_t *count;  // the view's tiles, stride words apart
+    uint32_t stride;
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &, uint32_t) const
+    {
+        atomicAdd(count + tile * stride, 1u);
+    }
+};
+
+struct ScatterPut {
+    uint32_t *slot;
+    uint32_t stride;
+    unsigned long long *words;
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t) const
+    {
+        words[atomicAdd(slot + tile * stride, 1u)] = ((unsigned long long)s.z << 32) | s.idx;
+    }
+};
+
+// The same for the pairs that fit the capacity only, in the ranges' ends;
+// without words they are only counted.
+struct CutPut {
+    ListState cut;
+    uint2 *ranges;
+    unsigned long long *words;
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t i) const
+    {
+        if (!pair_kept(cut, s, i)) return;
+        const uint32_t pos = atomicAdd(&ranges[tile].y, 1u);
+        if (words) words[pos] = ((unsigned long long)s.z << 32) | s.idx;
+    }
+};
+
+// The walk over all pairs of view v: put for each kept tile of a record's
+// rectangle.  Warps take granules of 32 records, warp
+// `first` of `stride`: drawn records come in runs (the map is in spatial order),
+// so granules far apart go to one warp and every warp gets a share of a run.
+// A lane walks its record's mask alone up to four tiles; larger records are
+// walked by half a warp, a tile a lane.
+template <bool DEPTH, typename PUT>
+__device__ __forceinline__ void walk_view(const ListArgs &a, const ViewInfo &V, uint32_t v, uint32_t first,
+                                          uint32_t stride, PUT put)
+{
+    constexpr int kAhead = 4;  // granules whose counts are loaded together
+    const int lane = threadIdx.x & 31;
+    const uint32_t granules = (a.n + 31) / 32;
+    const size_t rbase = (size_t)v * a.n;
+    const uint32_t tiles_x = (uint32_t)V.tiles_x;
+    for (uint64_t g0 = first; g0 < granules; g0 += (uint64_t)kAhead * stride) {
+        uint32_t cnt[kAhead];
+        #pragma unroll
+        for (int k = 0; k < kAhead; k++) {
+            const uint64_t i = (g0 + (uint64_t)k * stride) * 32 + lane;
+            cnt[k] = i < a.n ? a.tt[rbase + i] : 0u;
+        }
+        #pragma unroll 1
+        for (int k = 0; k < kAhead; k++) {
+            const uint32_t c = k == 0 ? cnt[0] : k == 1 ? cnt[1] : k == 2 ? cnt[2] : cnt[3];
+            if (!__any_sync(kFullMask, c > 0)) continue;
+            Splat s = {};
+            s.idx = (uint32_t)((g0 + (uint64_t)k * stride) * 32) + lane;
+            s.rbase = (uint32_t)rbase;
+            if (c) {
+                const size_t r = rbase + s.idx;
+                const uint2 rr = a.rect[r];
+                s.mask = a.mask[r];
+                s.z = DEPTH ? __float_as_uint(a.rec[12 * r + 2]) : 0u;
+                s.tile0 = (rr.x >> 16) * tiles_x + (rr.x & 0xffffu);
+                s.wh = ((rr.y & 0xffffu) - (rr.x & 0xffffu) + 1) | (((rr.y >> 16) - (rr.x >> 16) + 1) << 16);
+            }
+            const uint32_t w = s.wh & 0xffffu;
+            const uint32_t recip = c ? (65536u + w - 1) / w : 0u;  // i / w = i * recip >> 16 for i < 64
+            const bool alone = c > 0 && c <= 4 && w * (s.wh >> 16) <= 64;
+            if (alone) {
+                unsigned long long m = s.mask;
+                while (m) {
+                    const uint32_t i = (uint32_t)__ffsll((long long)m) - 1u;
+                    m &= m - 1ull;
+                    const uint32_t ky = (i * recip) >> 16;
+                    put(s.tile0 + ky * tiles_x + (i - ky * w), s, i);
+                }
+            }
+            // two of the larger records at a time, half a warp each
+            uint32_t todo = __ballot_sync(kFullMask, c > 0 && !alone);
+            while (todo) {
+                const int s0 = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const int s1 = __ffs(todo) - 1;  // -1: none
+                todo &= todo - 1;
+                const int src = lane < 16 ? s0 : s1;
+                const bool have = src >= 0;
+                Splat q;
+                q.rbase = s.rbase;
+                q.tile0 = __shfl_sync(kFullMask, s.tile0, src & 31);
+                q.wh = __shfl_sync(kFullMask, s.wh, src & 31);
+                q.mask = __shfl_sync(kFullMask, s.mask, src & 31);
+                const uint32_t inv = __shfl_sync(kFullMask, recip, src & 31);
+                q.z = DEPTH ? __shfl_sync(kFullMask, s.z, src & 31) : 0u;
+                q.idx = DEPTH ? __shfl_sync(kFullMask, s.idx, src & 31) : 0u;
+                const uint32_t qw = q.wh & 0xffffu, tiles = have ? qw * (q.wh >> 16) : 0u;
+                for (uint32_t i = lane & 15; i < tiles; i += 16) {
+                    const uint32_t ky = tiles <= 64 ? (i * inv) >> 16 : i / qw;
+                    if (tiles > 64 || ((q.mask >> i) & 1ull)) put(q.tile0 + ky * tiles_x + (i - ky * qw), q, i);
+                }
+                __syncwarp();
+            }
+        }
+    }
+}
+
+// One block of kScanThreads: the tile counts (ranges[t].y) to each tile's
+// [start, end) ([0, 0) when empty), the long tiles' chunks to the list.  With
+// `advance` the end is left at the start, for a scatter that moves it on.
+// Returns the total; the ranges are complete only when it fits.
+__device__ __forceinline__ uint64_t scan_tiles(const ListArgs &a, uint32_t n_tiles, bool advance)
+{
+    constexpr int kPer = 4;
+    __shared__ uint64_t tmp[32];
+    __shared__ uint32_t s_long;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_long = 0;
+    uint64_t carry = 0;
+    uint32_t c[kPer], next[kPer];
+    auto load = [&](uint32_t t0, uint32_t (&x)[kPer]) {
+        #pragma unroll
+        for (int k = 0; k < kPer; k++) {
+            const uint32_t t = t0 + threadIdx.x * kPer + k;
+            x[k] = t < n_tiles ? a.ranges[t].y : 0u;
+        }
+    };
+    load(0, c);
+    for (uint32_t t0 = 0; t0 < n_tiles; t0 += kScanThreads * kPer) {
+        load(t0 + kScanThreads * kPer, next);
+        uint64_t x = 0;
+        #pragma unroll
+        for (int k = 0; k < kPer; k++) x += c[k];
+        uint64_t inc = x;
+        #pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(kFullMask, inc, o);
+            if (lane >= o) inc += y;
+        }
+        __syncthreads();  // the last round's sums have been read
+        if (lane == 31) tmp[warp] = inc;
+        __syncthreads();
+        const uint64_t w = tmp[lane];  // every warp scans the warps' sums
+        uint64_t wi = w;
+        #pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(kFullMask, wi, o);
+            if (lane >= o) wi += y;
+        }
+        uint64_t at = carry + __shfl_sync(kFullMask, wi - w, warp) + inc - x;
+        carry += __shfl_sync(kFullMask, wi, 31);
+        #pragma unroll
+        for (int k = 0; k < kPer; k++) {
+            const uint32_t t = t0 + threadIdx.x * kPer + k;
+            if (t < n_tiles && c[k] && at + c[k] <= a.cap) {
+                a.ranges[t] = make_uint2((uint32_t)at, (uint32_t)(advance ? at : at + c[k]));
+                if (c[k] > kGroupWords) {
+                    const uint32_t chunks = (c[k] + kTileChunk - 1) / kTileChunk;
+                    const uint32_t slot = atomicAdd(&s_long, chunks);
+                    for (uint32_t j = 0; j < chunks; j++) a.long_chunks[slot + j] = make_uint2(t, j);
+                }
+            }
+            at += c[k];
+            c[k] = next[k];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) a.state->n_long = s_long;
+    return carry;
+}
+
+// One block, only when the pairs exceed the capacity: the (depth, record id)
+// up to which the nearest records' pairs fit, by a radix selection over all
+// drawn records weighted by their pairs (11 bits a pass), then the counts of
+// the pairs that stay.  Rare and slow (one block reads all records).
+__device__ __noinline__ void cut_to_capacity(const ListArgs &a, const ViewTable &vt, uint32_t n_tiles)
+{
+    constexpr int kBits = 11, kBins = 1 << kBits;
+    __shared__ unsigned long long hist[kBins];
+    __shared__ unsigned long long s_prefix, s_room;
+    if (threadIdx.x == 0) {
+        s_prefix = 0;
+        s_room = a.cap;
+    }
+    for (int shift = 55; shift >= 0; shift -= kBits) {  // 64 bits: digits at 55 (9 bits), 44, 33, 22, 11, 0
+        for (int k = threadIdx.x; k < kBins; k += kScanThreads) hist[k] = 0;
+        __syncthreads();
+        const unsigned long long prefix = s_prefix;
+        #pragma unroll 4
+        for (uint64_t r = threadIdx.x; r < a.total; r += kScanThreads) {
+            const uint32_t c = a.tt[r];
+            if (!c) continue;
+            const unsigned long long key =
+                ((unsigned long long)__float_as_uint(a.rec[12 * r + 2]) << 32) | (unsigned long long)r;
+            if (shift == 55 || (key >> (shift + kBits)) == (prefix >> (shift + kBits)))
+                atomicAdd(&hist[(key >> shift) & (kBins - 1)], (unsigned long long)c);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned long long room = s_room;
+            int d = 0;
+            while (d < kBins - 1 && hist[d] <= room) room -= hist[d++];
+            s_room = room;
+            s_prefix = prefix | ((unsigned long long)d << shift);
+        }
+        __syncthreads();
+    }
+    const ListState cut = {0u, 1u, (uint32_t)(s_prefix >> 32), (uint32_t)s_prefix, (uint32_t)s_room};
+    if (threadIdx.x == 0) *a.state = cut;
+    for (uint32_t t = threadIdx.x; t < n_tiles; t += kScanThreads) a.ranges[t] = make_uint2(0u, 0u);
+    __threadfence();
+    __syncthreads();
+    for (int v = 0; v < vt.n_views; v++)
+        walk_view<true>(a, vt.v[v], v, threadIdx.x / 32, kScanThreads / 32,
+                        CutPut{cut, a.ranges + vt.v[v].tile_base, nullptr});
+    __threadfence();
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(ListArgs a, ViewTable vt, bool advance)
+{
+    const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
+    if (threadIdx.x == 0) *a.state = ListState{};
+    const uint64_t pairs = scan_tiles(a, n_tiles, advance);
+    if (threadIdx.x == 0) {
+        *a.n_pairs = pairs > 0xffffffffull ? 0xffffffffu : (uint32_t)pairs;
+        if (pairs > a.cap) raise_status(a.status, GS_ERR_CAPACITY);
+    }
+    if (pairs > a.cap) {  // block-uniform
+        __syncthreads();
+        cut_to_capacity(a, vt, n_tiles);
+        scan_tiles(a, n_tiles, true);
+    }
+}
+
+// Grid: blocks of view 0, of view 1, ...  PRIVATE: a block counts its view's
+// tiles in shared memory and adds them up at the end; the sum that an addition
+// finds is the block's first slot in that tile's list, kept in its row of the
+// table for the scatter.  (On the tiles' global words directly, the additions of
+// a 60,000-word tile wait for one another: 1.2 ms on a 4M-Gaussian floor.)
+// Without, the additions are global ones: for small maps, where a table row a
+// block would not fit the workspace.
+template <bool PRIVATE>
+__global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_count_kernel(ListArgs a, ViewTable vt, uint32_t blocks_per_view)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    uint32_t *s_tile = reinterpret_cast<uint32_t *>(s_raw);  // the view's tiles
+    const uint32_t v = blockIdx.x / blocks_per_view, b = blockIdx.x - v * blocks_per_view;
+    const ViewInfo &V = vt.v[v];
+    const uint32_t tiles = (uint32_t)(V.tiles_x * V.tiles_y);
+    uint2 *ranges = a.ranges + V.tile_base;
+    if (PRIVATE) {
+        for (uint32_t t = threadIdx.x; t < tiles; t += kListThreads) s_tile[t] = 0;
+        __syncthreads();
+    }
+    walk_view<false>(a, V, v, b * (kListThreads / 32) + threadIdx.x / 32, blocks_per_view * (kListThreads / 32),
+                     PRIVATE ? CountPut{s_tile, 1u} : CountPut{&ranges[0].y, 2u});
+    if (PRIVATE) {
+        __syncthreads();
+        uint32_t *row = a.table + (size_t)blockIdx.x * a.table_pitch;
+        // four additions in flight a thread; the blocks start at different
+        // tiles, so that they do not queue for the same words
+        const uint32_t start = (uint32_t)(((uint64_t)tiles * b) / blocks_per_view);
+        for (uint32_t t0 = threadIdx.x; t0 < tiles; t0 += 4 * kListThreads) {
+            uint32_t t[4], c[4];
+            #pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const uint32_t u = t0 + k * kListThreads;
+                t[k] = u + start < tiles ? u + start : u + start - tiles;
+                c[k] = u < tiles ? s_tile[t[k]] : 0u;
+            }
+            #pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const uint32_t n = c[k];
+                if (n) c[k] = atomicAdd(&ranges[t[k]].y, n);
+                t[k] = n ? t[k] : ~0u;
+            }
+            #pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (t[k] != ~0u) row[t[k]] = c[k];
+        }
+    }
+}
+
+// The same grid and walk: each pair to its tile's next slot, from the block's
+// first slot in shared memory (PRIVATE) or the tile's end in the ranges (which
+// then advances to the list's end).
+template <bool PRIVATE>
+__global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_scatter_kernel(ListArgs a, ViewTable vt, uint32_t blocks_per_view)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    uint32_t *s_tile = reinterpret_cast<uint32_t *>(s_raw);
+    const uint32_t v = blockIdx.x / blocks_per_view, b = blockIdx.x - v * blocks_per_view;
+    const ViewInfo &V = vt.v[v];
+    const uint32_t tiles = (uint32_t)(V.tiles_x * V.tiles_y);
+    uint2 *ranges = a.ranges + V.tile_base;
+    const ListState st = *a.state;
+    const uint32_t first = b * (kListThreads / 32) + threadIdx.x / 32, stride = blocks_per_view * (kListThreads / 32);
+    if (PRIVATE && !st.cut) {
+        // (rows are written only where the block has pairs: other slots are not used)
+        const uint32_t *row = a.table + (size_t)blockIdx.x * a.table_pitch;
+        #pragma unroll 4
+        for (uint32_t t = threadIdx.x; t < tiles; t += kListThreads) s_tile[t] = ranges[t].x + row[t];
+        __syncthreads();
+        walk_view<true>(a, V, v, first, stride, ScatterPut{s_tile, 1u, a.words});
+    } else if (!st.cut) {
+        walk_view<true>(a, V, v, first, stride, ScatterPut{&ranges[0].y, 2u, a.words});
+    } else {
+        walk_view<true>(a, V, v, first, stride, CutPut{st, ranges, a.words});
+    }
+}
+
+// Ascending bitonic sort of a warp's 32 PER words, word lane * PER + r in
+// register r of a lane: strides below PER stay in the lane.
+template <int PER>
+__device__ __forceinline__ void warp_sort(unsigned long long (&k)[PER], int lane)
+{
+    #pragma unroll
+    for (int size = 2; size <= 32 * PER; size <<= 1) {
+        #pragma unroll
+        for (int stride = size / 2; stride > 0; stride >>= 1) {
+            if (stride >= PER) {
+                const int ls = stride / PER;
+                const bool low = (lane & ls) == 0;
+                const bool up = size >= 32 * PER || ((lane * PER) & size) == 0;
+                #pragma unroll
+                for (int r = 0; r < PER; r++) {
+                    const unsigned long long o = __shfl_xor_sync(kFullMask, k[r], ls);
+                    k[r] = (k[r] < o) == (low == up) ? k[r] : o;
+                }
+            } else {
+                #pragma unroll
+                for (int r = 0; r < PER; r++) {
+                    if (r & stride) continue;
+                    const bool up = size >= 32 * PER || ((size < PER ? r : lane * PER) & size) == 0;
+                    const unsigned long long x = k[r], y = k[r | stride];
+                    const bool swap = (x > y) == up;
+                    k[r] = swap ? y : x;
+                    k[r | stride] = swap ? x : y;
+                }
+            }
+        }
+    }
+}
+
+// Sorts words [0, m) of src, m <= THREADS PER, by THREADS threads: each warp a
+// run of 32 PER in registers, then rounds of merging by rank in shared memory.
+// s[0, m) holds the result; sync() is a barrier of the THREADS threads.
+template <int PER, int THREADS, typename SYNC>
+__device__ __forceinline__ void group_sort(const unsigned long long *src, uint32_t m, unsigned long long *s, int tid,
+                                           SYNC sync)
+{
+    constexpr uint32_t kRun = 32 * PER;
+    const int lane = tid & 31, warp = tid >> 5;
+    unsigned long long k[PER];
+    const uint32_t first = warp * kRun;
+    if (first < m) {
+        // coalesced loads; the order within the run does not matter
+        #pragma unroll
+        for (int r = 0; r < PER; r++) {
+            const uint32_t i = first + r * 32 + lane;
+            k[r] = i < m ? src[i] : ~0ull;
+        }
+        warp_sort<PER>(k, lane);
+    } else {
+        #pragma unroll
+        for (int r = 0; r < PER; r++) k[r] = ~0ull;
+    }
+    #pragma unroll
+    for (int r = 0; r < PER; r++) s[first + lane * PER + r] = k[r];
+    sync();
+    #pragma unroll 1
+    for (uint32_t run = kRun; run < m; run *= 2) {  // until one run holds every word (the rest is padding)
+        uint32_t to[PER];
+        #pragma unroll
+        for (int r = 0; r < PER; r++) {
+            const uint32_t p = r * THREADS + tid;
+            to[r] = ~0u;
+            k[r] = ~0ull;
+            if (p >= m) continue;  // padding: already behind every word
+            k[r] = s[p];
+            // words of the sibling run below this one
+            const uint32_t sib = (p & ~(run - 1)) ^ run;
+            uint32_t lo = 0;
+            for (uint32_t half = run >> 1; half > 0; half >>= 1) lo += s[sib + lo + half - 1] < k[r] ? half : 0u;
+            lo += s[sib + lo] < k[r] ? 1u : 0u;
+            to[r] = (p & ~(2 * run - 1)) + (p & (run - 1)) + lo;
+        }
+        sync();
+        #pragma unroll
+        for (int r = 0; r < PER; r++)
+            if (to[r] != ~0u) s[to[r]] = k[r];
+        sync();
+    }
+}
+
+// A block per listed chunk of a long tile (the first `extra` blocks), then four
+// tiles a block, 128 threads each with a barrier of their own.  A long tile of
+// one chunk is finished here; the chunks of longer ones go back sorted.
+__global__ void __launch_bounds__(kSortBlock, 2) tile_sort_kernel(ListArgs a, uint32_t n_tiles, uint32_t extra)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    unsigned long long *s = reinterpret_cast<unsigned long long *>(s_raw);
+    if (blockIdx.x < extra) {
+        const uint32_t n_long = a.state->n_long;
+        for (uint32_t j = blockIdx.x; j < n_long; j += extra) {
+            const uint2 tc = a.long_chunks[j];
+            const uint2 r = a.ranges[tc.x];
+            const uint32_t b = r.x + tc.y * kTileChunk, m = min(kTileChunk, r.y - b);
+            auto sync = []() { __syncthreads(); };
+            if (m <= 8 * kSortBlock) group_sort<8, kSortBlock>(a.words + b, m, s, threadIdx.x, sync);
+            else group_sort<16, kSortBlock>(a.words + b, m, s, threadIdx.x, sync);
+            const bool whole = r.y - r.x <= kTileChunk;
+            for (uint32_t i = threadIdx.x; i < m; i += kSortBlock) {
+                const unsigned long long w = s[i];
+                if (whole) {
+                    a.keys[b + i] = ((uint64_t)tc.x << 32) | (w >> 32);
+                    a.vals[b + i] = (uint32_t)w;
+                } else {
+                    a.words[b + i] = w;
+                }
+            }
+            __syncthreads();
+        }
+        return;
+    }
+    const int group = threadIdx.x / kSortGroup, tid = threadIdx.x % kSortGroup;
+    const uint32_t tile = (blockIdx.x - extra) * (kSortBlock / kSortGroup) + group;
+    if (tile >= n_tiles) return;
+    const uint2 r = a.ranges[tile];
+    const uint32_t m = r.y - r.x;
+    if (m == 0 || m > kGroupWords) return;
+    s += group * kGroupWords;
+    const unsigned long long *src = a.words + r.x;
+    auto sync = [group]() { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(kSortGroup) : "memory"); };
+    if (m <= kSortGroup) group_sort<1, kSortGroup>(src, m, s, tid, sync);
+    else if (m <= 2 * kSortGroup) group_sort<2, kSortGroup>(src, m, s, tid, sync);
+    else if (m <= 4 * kSortGroup) group_sort<4, kSortGroup>(src, m, s, tid, sync);
+    else if (m <= 8 * kSortGroup) group_sort<8, kSortGroup>(src, m, s, tid, sync);
+    else group_sort<16, kSortGroup>(src, m, s, tid, sync);
+    for (uint32_t i = tid; i < m; i += kSortGroup) {
+        const unsigned long long w = s[i];
+        a.keys[r.x + i] = ((uint64_t)tile << 32) | (w >> 32);
+        a.vals[r.x + i] = (uint32_t)w;
+    }
+}
+
+// Each word of a listed chunk goes to its rank in the tile: its place in its
+// own chunk plus the words below it in the tile's other chunks.
+__global__ void __launch_bounds__(kMergeThreads) tile_merge_kernel(ListArgs a)
+{
+    const uint32_t n_long = a.state->n_long;
+    for (uint32_t j = blockIdx.x; j < n_long; j += gridDim.x) {
+        const uint2 tc = a.long_chunks[j];
+        const uint2 r = a.ranges[tc.x];
+        const uint32_t m = r.y - r.x, chunks = (m + kTileChunk - 1) / kTileChunk;
+        if (chunks == 1) continue;  // finished by the sort
+        const unsigned long long *w = a.words + r.x;
+        const uint32_t lo0 = tc.y * kTileChunk, hi0 = min(m, lo0 + kTileChunk);
+        for (uint32_t i = lo0 + threadIdx.x; i < hi0; i += kMergeThreads) {
+            const unsigned long long x = w[i];
+            uint32_t rank = i - lo0;
+            for (uint32_t c = 0; c < chunks; c++) {
+                if (c == tc.y) continue;
+                const unsigned long long *run = w + c * kTileChunk;
+                uint32_t lo = 0, n = min(kTileChunk, m - c * kTileChunk);
+                while (n > 0) {
+                    const uint32_t half = n >> 1;
+                    const bool below = run[lo + half] < x;
+                    lo = below ? lo + half + 1 : lo;
+                    n = below ? n - half - 1 : half;
+                }
+                rank += lo;
+            }
+            a.keys[r.x + rank] = ((uint64_t)tc.x << 32) | (x >> 32);
+            a.vals[r.x + rank] = (uint32_t)x;
+        }
+    }
+}
+
+template <bool PRIVATE>
+static gs_status_t launch_walks(const ListArgs &a, const ViewTable &vt, uint32_t blocks_per_view, size_t smem,
+                                cudaStream_t s)
+{
+    const unsigned grid = blocks_per_view * (unsigned)vt.n_views;
+    if (smem > 48 * 1024) {
+        const cudaFuncAttribute most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        if (cudaFuncSetAttribute(tile_count_kernel<PRIVATE>, most, (int)smem) != cudaSuccess ||
+            cudaFuncSetAttribute(tile_scatter_kernel<PRIVATE>, most, (int)smem) != cudaSuccess)
+            return GS_ERR_CUDA;
+    }
+    tile_count_kernel<PRIVATE><<<grid, kListThreads, smem, s>>>(a, vt, blocks_per_view);
+    tile_scan_kernel<<<1, kScanThreads, 0, s>>>(a, vt, !PRIVATE);
+    tile_scatter_kernel<PRIVATE><<<grid, kListThreads, smem, s>>>(a, vt, blocks_per_view);
+    return launch_status();
+}
+
+// Where a tile's list could grow very long, its chunks' merge (a search in
+// every other chunk) would cost more than the radix passes: the records per
+// tile decide, since the host knows no pair counts.  At 2,000 records a tile
+// (950k Gaussians, four views of 400x304) whole mapping steps took 1,385
+// against 1,522 us with the radix path (a room), 1,677 against 1,776 (a long
+// floor, the lists most uneven); 200k Gaussians on 176x144: renders of 126
+// against 193 us and 222 against 272.  The scan of the tiles is one block's,
+// hence the limit on their number.
+bool tile_lists_fit(int64_t n_records, int64_t n_tiles)
+{
+    return n_records <= 2048 * n_tiles && n_tiles <= (int64_t(1) << 18);
+}
+
+gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, const ViewTable &vt, gs_bins_t *bins,
+                       const TileListBuffers &buf, cudaStream_t s)
+{
+    ListArgs a;
+    a.rec = proj->rec;
+    a.rect = reinterpret_cast<const uint2 *>(proj->rect);
+    a.mask = reinterpret_cast<const unsigned long long *>(proj->tile_mask);
+    a.tt = proj->tiles_touched;
+    a.total = (uint32_t)total;
+    a.n = (uint32_t)n;
+    a.cap = (uint32_t)bins->capacity;
+    a.ranges = reinterpret_cast<uint2 *>(bins->ranges);
+    a.n_pairs = bins->n_pairs;
+    a.status = bins->status;
+    a.state = reinterpret_cast<ListState *>(buf.small);
+    a.long_chunks = static_cast<uint2 *>(buf.chunks);
+    a.words = static_cast<unsigned long long *>(buf.words);
+    a.keys = bins->keys;
+    a.vals = bins->vals;
+    const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
+    if (cudaMemsetAsync(a.ranges, 0, sizeof(uint2) * (size_t)n_tiles, s) != cudaSuccess) return GS_ERR_CUDA;
+    uint32_t most_tiles = 0;
+    for (int v = 0; v < vt.n_views; v++) {
+        const uint32_t t = (uint32_t)(vt.v[v].tiles_x * vt.v[v].tiles_y);
+        most_tiles = t > most_tiles ? t : most_tiles;
+    }
+    // blocks a view: a granule of 32 records a warp at least, a few waves at
+    // most (views differ in what they see: with one wave the fullest view's
+    // blocks finish last, 420 against 300 us on a 4M-Gaussian floor)
+    const int64_t wanted = (n + kListThreads - 1) / kListThreads;
+    const int64_t slots = (int64_t)num_sms() * 4 * kBlocksPerSm / vt.n_views;
+    int64_t per_view = wanted < slots ? wanted : slots;
+    const size_t smem = sizeof(uint32_t) * most_tiles;
+    const int64_t rows = (int64_t)(buf.table_bytes / smem) / vt.n_views;  // table rows a view
+    const bool priv = smem <= kMaxTileSmem && (rows >= per_view || rows * vt.n_views >= num_sms());
+    gs_status_t st;
+    if (priv) {
+        per_view = per_view < rows ? per_view : rows;
+        a.table = static_cast<uint32_t *>(buf.table);
+        a.table_pitch = most_tiles;
+        st = launch_walks<true>(a, vt, (uint32_t)per_view, smem, s);
+    } else {
+        a.table = nullptr;
+        a.table_pitch = 0;
+        st = launch_walks<false>(a, vt, (uint32_t)per_view, 0, s);
+    }
+    if (st != GS_OK) return st;
+    const uint32_t extra = (uint32_t)num_sms() * 2;
+    const size_t sort_smem = sizeof(unsigned long long) * kTileChunk;
+    if (cudaFuncSetAttribute(tile_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem) != cudaSuccess)
+        return GS_ERR_CUDA;
+    const unsigned groups = kSortBlock / kSortGroup;
+    tile_sort_kernel<<<(n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s>>>(a, n_tiles, extra);
+    tile_merge_kernel<<<(unsigned)num_sms() * 8, kMergeThreads, 0, s>>>(a);
+    return launch_status();
+}
+
+}  // namespace gs

@@ -206,10 +206,14 @@ class MappingStep:
 
     def kernels_per_step(self):
         """Kernels of this library launched by one run() (memsets excluded)."""
-        # bin: record count, scan, compaction, 4 depth passes, pair count, scan, emission, the tile-id
-        # passes (8 bits each) and the ranges
-        tile_passes = max(1, (max(self.rast.n_tiles - 1, 0).bit_length() + 7) // 8)
-        k_bin = 3 + 4 + 3 + tile_passes + 1
+        r = self.rast
+        if r.n * r.V <= 2048 * r.n_tiles and r.n_tiles <= 1 << 18:
+            k_bin = 5  # tile count, scan, scatter, sort, merge
+        else:
+            # record count, scan, compaction, 4 depth passes, pair count, scan, emission, the tile-id
+            # passes (8 bits each) and the ranges
+            tile_passes = max(1, (max(r.n_tiles - 1, 0).bit_length() + 7) // 8)
+            k_bin = 3 + 4 + 3 + tile_passes + 1
         # project, bin, fwd (with the L1 loss), bwd, pbwd colour + geometry
         k = 1 + k_bin + 1 + 1 + 2
         k += 2 if self.zeta > 0 else 0
