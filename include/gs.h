@@ -254,7 +254,7 @@ gs_status_t gs_bin_sort_noalloc(const gs_projected_t *proj, int64_t n, const gs_
  * alpha_i = min(0.99, o_i exp(-1/2 d^T conic d)); entries with alpha < 1/255
  * are skipped; compositing stops before an entry that would bring T below
  * 1e-4.  One persistent launch over all (view, tile) work items.
- * work_counter: device uint32 scratch, reset inside the call. */
+ * work_counter: device uint32 scratch, reset inside the call when it is used. */
 gs_status_t gs_render_fwd(const gs_projected_t *proj, int64_t n, const gs_bins_t *bins,
                           const gs_view_t *views, int32_t n_views, gs_image_t *img,
                           uint32_t *work_counter, void *stream);
@@ -287,7 +287,8 @@ gs_status_t gs_render_stats(const gs_projected_t *proj, int64_t n, const gs_bins
  * a view's tile falls back to the (2, 8) band of the same staging; defaults:
  * forward 7, backward 9, the asynchronous-copy (2, 8) and (4, 8)).  All
  * variants compute the same result; the autotuner times them on the workload
- * and sets the fastest.  The setting is process-wide and read when a kernel
+ * and sets the fastest.  Until they are set, images of few pixels take the
+ * (1, 8) and (2, 8) bands of the default staging.  The setting is process-wide and read when a kernel
  * is launched.  GS_ERR_INVALID_ARG for an index out of range. */
 gs_status_t gs_set_render_variants(int32_t fwd, int32_t bwd);
 

@@ -381,6 +381,16 @@ class Rasterizer:
         self.generation += 1
         return self.img
 
+    def forward_l1(self, params, viewmats, target_rgb, target_depth, w_c, w_d, use_gate, gamma, loss, d_rgb, d_depth,
+                   stream=None):
+        """forward with gs_loss_l1 evaluated on each pixel as it finishes."""
+        gs_project(params, self.views, viewmats, self.proj, self.near_z, self.blur, stream)
+        gs_bin_sort(self.proj, self.n, self.views, self.bins, self.workspace, stream)
+        gs_render_fwd_l1(self.proj, self.n, self.bins, self.views, self.img, self.work_counter, target_rgb,
+                         target_depth, w_c, w_d, use_gate, gamma, loss, d_rgb, d_depth, stream)
+        self.generation += 1
+        return self.img
+
     def backward(self, params, viewmats, d_rgb, d_depth, d_alpha, grads, d_twist=None, stream=None,
                  overwrite_grads=False):
         """Accumulate parameter gradients (or write them, with

@@ -68,47 +68,44 @@ __global__ void __launch_bounds__(256) adam_kernel(float *__restrict__ param, co
 }
 
 // E <- Exp(xi) E, xi <- 0 (xi = (rho, phi); closed-form SE(3) exponential).
-__global__ void pose_update_kernel(float *viewmats, float *twist, int n_views)
+// Twelve lanes a view, an entry of [R | t] each.  Bound: the latency of FP64
+// arithmetic (few units on this GPU), so the entries are computed side by side
+// and, below 0.1 rad, A = sin th / th, B = (1 - cos th) / th^2 and C =
+// (th - sin th) / th^3 by their series in th^2 (five terms: the next is below
+// 1e-17) instead of sine, cosine and quotients.  One thread a view took 9.0 us.
+__global__ void __launch_bounds__(32) pose_update_kernel(float *viewmats, float *twist)
 {
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n_views) return;
-    double rho[3], ph[3];
-    for (int k = 0; k < 3; k++) {
-        rho[k] = twist[6 * v + k];
-        ph[k] = twist[6 * v + 3 + k];
-    }
-    const double th2 = ph[0] * ph[0] + ph[1] * ph[1] + ph[2] * ph[2], th = sqrt(th2);
+    const int v = blockIdx.x, e = threadIdx.x;
+    const int i = e < 12 ? e >> 2 : 0, j = e & 3;
+    float *E = viewmats + 12 * v, *xi = twist + 6 * v;
+    const double rho[3] = {xi[0], xi[1], xi[2]}, ph[3] = {xi[3], xi[4], xi[5]};
+    const double th2 = ph[0] * ph[0] + ph[1] * ph[1] + ph[2] * ph[2];
     double A, B, C;
-    if (th < 1e-5) {
-        A = 1.0 - th2 / 6.0;
-        B = 0.5 - th2 / 24.0;
-        C = 1.0 / 6.0 - th2 / 120.0;
+    if (th2 < 1e-2) {
+        A = 1.0 - th2 * (1.0 / 6 - th2 * (1.0 / 120 - th2 * (1.0 / 5040 - th2 * (1.0 / 362880))));
+        B = 0.5 - th2 * (1.0 / 24 - th2 * (1.0 / 720 - th2 * (1.0 / 40320 - th2 * (1.0 / 3628800))));
+        C = 1.0 / 6 - th2 * (1.0 / 120 - th2 * (1.0 / 5040 - th2 * (1.0 / 362880 - th2 * (1.0 / 39916800))));
     } else {
+        const double th = sqrt(th2);
         A = sin(th) / th;
         B = (1.0 - cos(th)) / th2;
         C = (th - sin(th)) / (th2 * th);
     }
-    const double Kx[3][3] = {{0, -ph[2], ph[1]}, {ph[2], 0, -ph[0]}, {-ph[1], ph[0], 0}};
-    double K2[3][3], R[3][3], Vm[3][3], t[3];
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) K2[i][j] = Kx[i][0] * Kx[0][j] + Kx[i][1] * Kx[1][j] + Kx[i][2] * Kx[2][j];
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) {
-            const double I = i == j ? 1.0 : 0.0;
-            R[i][j] = I + A * Kx[i][j] + B * K2[i][j];
-            Vm[i][j] = I + B * Kx[i][j] + C * K2[i][j];
-        }
-    for (int i = 0; i < 3; i++) t[i] = Vm[i][0] * rho[0] + Vm[i][1] * rho[1] + Vm[i][2] * rho[2];
-    float *E = viewmats + 12 * v;
-    double out[12];
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 4; j++) {
-            double acc = R[i][0] * E[j] + R[i][1] * E[4 + j] + R[i][2] * E[8 + j];
-            if (j == 3) acc += t[i];
-            out[4 * i + j] = acc;
-        }
-    for (int k = 0; k < 12; k++) E[k] = (float)out[k];
-    for (int k = 0; k < 6; k++) twist[6 * v + k] = 0.0f;
+    // row i of K = [ph]x, K^2 = ph ph^T - th2 I, R = I + A K + B K^2, V = I + B K + C K^2
+    const double p0 = ph[0], p1 = ph[1], p2 = ph[2];
+    const double k[3] = {i == 0 ? 0.0 : i == 1 ? p2 : -p1, i == 0 ? -p2 : i == 1 ? 0.0 : p0,
+                         i == 0 ? p1 : i == 1 ? -p0 : 0.0};
+    const double pi = i == 0 ? p0 : i == 1 ? p1 : p2;
+    double out = 0.0;
+    #pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const double I = i == c ? 1.0 : 0.0, k2 = pi * ph[c] - th2 * I;
+        out += (I + A * k[c] + B * k2) * (double)E[4 * c + j];
+        if (j == 3) out += (I + B * k[c] + C * k2) * rho[c];
+    }
+    __syncwarp();  // every entry of the old pose and the twist has been read
+    if (e < 12) E[e] = (float)out;
+    if (e < 6) xi[e] = 0.0f;
 }
 
 }  // namespace gs
@@ -145,6 +142,6 @@ extern "C" gs_status_t gs_adam_step(float *param, const float *grad, float *m, f
 extern "C" gs_status_t gs_pose_update(float *viewmats, float *twist, int32_t n_views, void *stream)
 {
     if (!viewmats || !twist || n_views < 1 || n_views > GS_MAX_VIEWS) return GS_ERR_INVALID_ARG;
-    pose_update_kernel<<<1, 64, 0, as_stream(stream)>>>(viewmats, twist, n_views);
+    pose_update_kernel<<<n_views, 32, 0, as_stream(stream)>>>(viewmats, twist);
     return launch_status();
 }

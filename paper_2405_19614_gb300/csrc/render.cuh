@@ -170,8 +170,8 @@ constexpr int kBwdVariants = 4 * kBandVariants;
 inline bool variant_gathers(int var) { return var >= 2 * kBandVariants; }
 constexpr int kVariantPPT[kBandVariants] = {1, 2, 2, 4, 4, 8};
 constexpr int kVariantBW[kBandVariants] = {8, 8, 16, 8, 16, 16};
-int render_variant_fwd();
-int render_variant_bwd();
+int render_variant_fwd(int64_t n_pix);
+int render_variant_bwd(int64_t n_pix);
 
 // The variant a launch uses: var when its band divides the tile of every view,
 // else the (2, 8) band (8 x 8 pixels, which divides every allowed tile) with

@@ -56,7 +56,7 @@ struct RenderBwdArgs {
     const uint32_t *n_contrib;
     const float *d_rgb, *d_depth, *d_alpha;
     float *grad2d;
-    uint32_t *work_counter;
+    uint32_t *work_counter;  // null: the warps take the items in order, one each
     uint32_t *status;  // device error word (a bounded wait that expired), may be null
     uint32_t n_items;  // (view, tile, band) work items, set by the launcher
 };
@@ -148,10 +148,14 @@ __global__ void __launch_bounds__(kRenderThreads, RenderOccupancy<PPT, TMA || AS
         __syncwarp();
     }
     const int red_entry = lane / kPairs, red_pair = lane % kPairs;  // the row this lane adds up
-    for (;;) {
+    for (uint32_t turn = 0;; turn++) {
         uint32_t wi = 0;
-        if (lane == 0) wi = atomicAdd(a.work_counter, 1u);
-        wi = __shfl_sync(kFullMask, wi, 0);
+        if (a.work_counter) {
+            if (lane == 0) wi = atomicAdd(a.work_counter, 1u);
+            wi = __shfl_sync(kFullMask, wi, 0);
+        } else {  // a warp an item: nothing to hand out
+            wi = turn == 0 ? blockIdx.x * WARPS + warp : a.n_items;
+        }
         if (wi >= a.n_items) break;
         // work item -> view, tile of the view, band of the tile
         const int v = view_of_item(vt, (int)wi);
@@ -566,6 +570,10 @@ static gs_status_t launch_bwd(RenderBwdArgs a, ViewTable vt, const CUtensorMap &
     const int64_t slots = (int64_t)num_sms() * (per_sm > 0 ? per_sm : 1);
     const int64_t blocks_needed = ((int64_t)a.n_items + kRenderThreads / 32 - 1) / (kRenderThreads / 32);
     const int grid = (int)(slots < blocks_needed ? slots : blocks_needed);
+    // every item has a warp of its own when the grid holds them all: no counter
+    // to clear and none to wait for (2 us less of a small image)
+    if (blocks_needed <= slots) a.work_counter = nullptr;
+    else if (cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
     kern<<<grid > 0 ? grid : 1, kRenderThreads, 0, s>>>(a, vt, map);
     return launch_status();
 }
@@ -622,11 +630,10 @@ extern "C" gs_status_t gs_render_bwd_splats(const gs_projected_t *proj, int64_t 
     a.status = bins->status;
     // the variant and, for the gathering variants, the record tensor map (a
     // gathering variant whose map cannot be made runs with lane loads)
-    int var = fitting_variant(vt, render_variant_bwd());
+    int var = fitting_variant(vt, render_variant_bwd(vt.n_pix_total));
     CUtensorMap map = {};
     if (variant_gathers(var) && make_record_map(reinterpret_cast<const float *>(a.rec), n * vt.n_views, &map) != GS_OK)
         var -= 2 * kBandVariants;
-    if (cudaMemsetAsync(work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
     const int base = var % kBandVariants;
     switch (var / kBandVariants) {
     case 0: return dispatch_bwd_band<32, false>(base, a, vt, map, s);

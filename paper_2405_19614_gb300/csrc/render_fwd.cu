@@ -31,7 +31,7 @@ struct RenderFwdArgs {
     float *rgb, *depth, *alpha, *final_T;
     uint32_t *n_contrib;
     uint32_t *n_eval, *n_blend;  // STATS variant only
-    uint32_t *work_counter;
+    uint32_t *work_counter;  // null: the warps take the items in order, one each
     uint32_t *status;  // device error word (a bounded wait that expired), may be null
     uint32_t n_items;  // (view, tile, band) work items, set by the launcher
     // LOSS variant only: the L1 terms of a6 evaluated as each pixel finishes
@@ -98,10 +98,14 @@ __global__ void __launch_bounds__(kRenderThreads, ASYNC ? RenderOccupancy<PPT, t
         }
         __syncwarp();
     }
-    for (;;) {
+    for (uint32_t turn = 0;; turn++) {
         uint32_t wi = 0;
-        if (lane == 0) wi = atomicAdd(a.work_counter, 1u);
-        wi = __shfl_sync(kFullMask, wi, 0);
+        if (a.work_counter) {
+            if (lane == 0) wi = atomicAdd(a.work_counter, 1u);
+            wi = __shfl_sync(kFullMask, wi, 0);
+        } else {  // a warp an item: nothing to hand out
+            wi = turn == 0 ? blockIdx.x * WARPS + warp : a.n_items;
+        }
         if (wi >= a.n_items) break;
         // work item -> view, tile of the view, band of the tile
         const int v = view_of_item(vt, (int)wi);
@@ -435,6 +439,10 @@ static gs_status_t launch_fwd(RenderFwdArgs a, ViewTable vt, const CUtensorMap &
     const int64_t slots = (int64_t)num_sms() * (per_sm > 0 ? per_sm : 1);
     const int64_t blocks_needed = ((int64_t)a.n_items + kRenderThreads / 32 - 1) / (kRenderThreads / 32);
     const int grid = (int)(slots < blocks_needed ? slots : blocks_needed);
+    // every item has a warp of its own when the grid holds them all: no counter
+    // to clear and none to wait for (2 us less of a small image)
+    if (blocks_needed <= slots) a.work_counter = nullptr;
+    else if (cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
     kern<<<grid > 0 ? grid : 1, kRenderThreads, 0, s>>>(a, vt, map);
     return launch_status();
 }
@@ -506,8 +514,7 @@ extern "C" gs_status_t gs_render_fwd(const gs_projected_t *proj, int64_t n, cons
     a.work_counter = work_counter;
     a.status = bins->status;
     CUtensorMap map = {};
-    const int var = prepare_fwd(a, vt, render_variant_fwd(), &map);
-    if (cudaMemsetAsync(work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
+    const int var = prepare_fwd(a, vt, render_variant_fwd(vt.n_pix_total), &map);
     return dispatch_fwd<false>(var, a, vt, map, s);
 }
 
@@ -548,8 +555,7 @@ extern "C" gs_status_t gs_render_fwd_l1(const gs_projected_t *proj, int64_t n, c
     a.d_rgb = d_rgb;
     a.d_depth = d_depth;
     CUtensorMap map = {};
-    const int var = prepare_fwd(a, vt, render_variant_fwd(), &map);
-    if (cudaMemsetAsync(work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
+    const int var = prepare_fwd(a, vt, render_variant_fwd(vt.n_pix_total), &map);
     return dispatch_fwd<false, true>(var, a, vt, map, s);
 }
 
@@ -563,7 +569,6 @@ extern "C" gs_status_t gs_render_stats(const gs_projected_t *proj, int64_t n, co
     if (st != GS_OK) return st;
     if (!bins->ranges || !bins->vals || (n > 0 && !proj->rec)) return GS_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    if (cudaMemsetAsync(work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
     RenderFwdArgs a = {};
     a.rec = reinterpret_cast<const float4 *>(proj->rec);
     a.n = n;
@@ -582,8 +587,32 @@ extern "C" gs_status_t gs_render_stats(const gs_projected_t *proj, int64_t n, co
 namespace gs {
 static int g_variant_fwd = 7;  // (2, 8) bands, asynchronous-copy staging
 static int g_variant_bwd = 9;  // (4, 8) bands, asynchronous-copy staging
-int render_variant_fwd() { return g_variant_fwd; }
-int render_variant_bwd() { return g_variant_bwd; }
+static bool g_variants_set = false;
+
+// Until variants are set, few pixels take smaller bands: where a launch has
+// fewer bands than the GPU holds warps, the longest list of one band is the
+// launch's time, and a band of fewer pixels walks its list faster.  The lines
+// are where both sides measured alike; with `held` warps of a 4-warp, 8-block
+// launch (4,864):
+//   forward, one pixel a thread below held / 2 bands of 32 (78k pixels): 216
+//     against 299 us on 43k pixels of crowded lists, 23 against 28 on 12k, 26
+//     and 26 on 71k, 26 against 22 on 106k;
+//   backward, one pixel below the same line: 45 against 91 us (four pixels) on
+//     64x48, 589 against 1,227 on 43k, 55 against 69 on 71k; two pixels below
+//     0.65 held bands of 64 (202k pixels): 40 against 42 us on 106k, 53 against
+//     50 on 254k.
+int render_variant_fwd(int64_t n_pix)
+{
+    const int64_t held = (int64_t)num_sms() * 32;
+    return !g_variants_set && n_pix / 32 <= held / 2 ? 6 : g_variant_fwd;
+}
+
+int render_variant_bwd(int64_t n_pix)
+{
+    const int64_t held = (int64_t)num_sms() * 32;
+    if (g_variants_set) return g_variant_bwd;
+    return n_pix / 32 <= held / 2 ? 6 : n_pix / 64 <= held * 13 / 20 ? 7 : g_variant_bwd;
+}
 }  // namespace gs
 
 extern "C" gs_status_t gs_set_render_variants(int32_t fwd, int32_t bwd)
@@ -591,6 +620,7 @@ extern "C" gs_status_t gs_set_render_variants(int32_t fwd, int32_t bwd)
     if (fwd < 0 || fwd >= kFwdVariants || bwd < 0 || bwd >= kBwdVariants) return GS_ERR_INVALID_ARG;
     g_variant_fwd = fwd;
     g_variant_bwd = bwd;
+    g_variants_set = true;
     return GS_OK;
 }
 

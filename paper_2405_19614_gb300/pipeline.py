@@ -13,7 +13,7 @@ from __future__ import annotations
 import numpy as np
 import torch
 
-from . import (Rasterizer, gs_adam_step, gs_loss_l1, gs_loss_ssim, gs_reproj_loss_grad, gs_ssim_workspace_size)
+from . import Rasterizer, gs_adam_step, gs_loss_ssim, gs_reproj_loss_grad, gs_ssim_workspace_size
 
 PARAM_ORDER = ("means", "log_scales", "quats", "opacity_logit", "sh")
 DEFAULT_LR = dict(means=1.6e-4, log_scales=5e-3, quats=1e-3, opacity_logit=5e-2, sh=2.5e-3)
@@ -242,7 +242,10 @@ class TrackingStep:
         self.target_rgb, self.target_depth = target_rgb, target_depth
         self.keypoints = keypoints
         self.twist = torch.zeros(V * 6, device=dev)
-        self.d_twist = torch.zeros(V * 6, device=dev)
+        # the loss and the twist gradients share one buffer, cleared by one fill a step
+        self.acc = torch.zeros(4 + 6 * V, device=dev)
+        self.loss = self.acc[0:1]
+        self.d_twist = self.acc[4:]
         self.m = torch.zeros(V * 6, device=dev)
         self.v = torch.zeros(V * 6, device=dev)
         self.step_count = torch.zeros(2, dtype=torch.int32, device=dev)
@@ -252,17 +255,15 @@ class TrackingStep:
         P = self.rast.n_pix
         self.d_rgb = torch.zeros(P, 3, device=dev)
         self.d_depth = torch.zeros(P, device=dev)
-        self.loss = torch.zeros(1, device=dev)
         self.w_rpj, self.w_c, self.w_d, self.gamma = float(w_rpj), float(w_c), float(w_d), float(gamma)
 
     def run(self, stream=None):
         from . import gs_pose_update, gs_render_bwd
         r = self.rast
-        self.d_twist.zero_()
-        self.loss.zero_()
-        r.forward(self.params, self.viewmats, stream)
-        gs_loss_l1(r.img["rgb"], r.img["depth"], r.img["alpha"], self.target_rgb, self.target_depth, self.w_c,
-                   self.w_d, True, self.gamma, self.loss, self.d_rgb, self.d_depth, stream)
+        self.acc.zero_()
+        # the compositing evaluates the L1 terms as each pixel finishes
+        r.forward_l1(self.params, self.viewmats, self.target_rgb, self.target_depth, self.w_c, self.w_d, True,
+                     self.gamma, self.loss, self.d_rgb, self.d_depth, stream)
         gs_render_bwd(self.params, r.views, self.viewmats, r.proj, r.bins, r.img, self.d_rgb, self.d_depth, None,
                       r.grad2d, None, self.d_twist, r.work_counter, r.near_z, r.blur, stream)
         if self.keypoints is not None:
