@@ -314,7 +314,9 @@ gs_status_t gs_loss_l1(const float *rgb, const float *depth, const float *alpha,
 gs_status_t gs_decode_keyframes(const uint8_t *rgb8, const uint16_t *depth16, int64_t n_pixels, float depth_scale,
                                 float *rgb, float *depth, void *stream);
 
-/* Bytes of workspace gs_loss_ssim needs for n_pixels (9 floats per pixel). */
+/* Bytes of workspace of gs_loss_ssim for n_pixels: 9 floats per pixel and an
+ * eighth more, for rows padded to 16 bytes.  (9 floats per pixel are enough;
+ * a slower pass then runs where a width is not a multiple of 4.) */
 size_t gs_ssim_workspace_size(int64_t n_pixels);
 
 /* SSIM term of the mapping loss (Sec. 3.4: L_m = (1 - zeta)(w4 L1(D) +
@@ -323,8 +325,8 @@ size_t gs_ssim_workspace_size(int64_t n_pixels);
  * window (sigma 1.5, normalised, zero padding), C1 = 0.01^2, C2 = 0.03^2.
  * Adds weight * (1 - mean SSIM) over all pixels and channels of the views to
  * *loss and its gradient to d_rgb [P,3] (+=, so it sums with gs_loss_l1's).
- * rgb, target_rgb [P,3] device; views host; workspace device, >=
- * gs_ssim_workspace_size(P) bytes, 16-byte aligned for the staged gradient
+ * rgb, target_rgb [P,3] device; views host; workspace device, >= 9 floats per
+ * pixel (see gs_ssim_workspace_size), 16-byte aligned for the staged gradient
  * pass (else a slower pass runs).  status: device error word, may be NULL; an
  * asynchronous copy that never completes sets bit GS_ERR_TIMEOUT there (the
  * bounded wait gives up, the affected tiles' gradients are missing). */
