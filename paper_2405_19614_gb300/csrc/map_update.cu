@@ -222,8 +222,9 @@ struct RowArrays {
 };
 
 constexpr int kRowThreads = 256;
-constexpr int kRowUnroll = 8;
-constexpr int kRowUnits = kRowThreads * kRowUnroll;  // units a block copies (at least one row)
+constexpr int kRowUnroll = 2;
+constexpr int kRowRounds = 4;
+constexpr int kRowUnits = kRowThreads * kRowUnroll * kRowRounds;  // units a block copies (at least one row)
 
 // Kept rows of one array, from row0 on, as a flat span of units: consecutive
 // threads copy consecutive units, kRowUnroll of them in flight a thread.
@@ -232,7 +233,7 @@ __device__ __forceinline__ void copy_rows(const int32_t *__restrict__ new_index,
                                           U *__restrict__ dst, int64_t row0, uint32_t rows, uint32_t units)
 {
     const uint64_t span = (uint64_t)rows * units;
-    for (uint64_t e0 = threadIdx.x; e0 < span; e0 += kRowUnits) {
+    for (uint64_t e0 = threadIdx.x; e0 < span; e0 += kRowThreads * kRowUnroll) {
         int64_t to[kRowUnroll];
         U v[kRowUnroll];
         #pragma unroll
@@ -248,10 +249,10 @@ __device__ __forceinline__ void copy_rows(const int32_t *__restrict__ new_index,
         }
         #pragma unroll
         for (int k = 0; k < kRowUnroll; k++)
-            if (to[k] >= 0) v[k] = src[(int64_t)units * row0 + (int64_t)(e0 + (uint64_t)k * kRowThreads)];
+            if (to[k] >= 0) v[k] = __ldcs(src + (int64_t)units * row0 + (int64_t)(e0 + (uint64_t)k * kRowThreads));
         #pragma unroll
         for (int k = 0; k < kRowUnroll; k++)
-            if (to[k] >= 0) dst[to[k]] = v[k];
+            if (to[k] >= 0) __stcs(dst + to[k], v[k]);
     }
 }
 
@@ -259,8 +260,9 @@ __device__ __forceinline__ void copy_rows(const int32_t *__restrict__ new_index,
 // and array).  A block copies a span of about 2,048 units of one array; rows
 // of a multiple of four floats move 16 bytes at a time.  A thread per row,
 // copying its row float by float, touched a 32-byte sector per 4-byte access:
-// 1,327 us for 15 arrays (SH3 parameters, m, v) of 1M rows, now 284 us
-// (1.42 GB, 5.0 TB/s).
+// 1,327 us for 15 arrays (SH3 parameters, m, v) of 1M rows, now 234 us
+// (1.42 GB, 6.1 TB/s; two units in flight a thread in four rounds, streaming
+// accesses; eight in flight in one round and cached took 284 us).
 __global__ void __launch_bounds__(kRowThreads) compact_rows_kernel(const int32_t *__restrict__ new_index, int64_t n,
                                                                    RowArrays A)
 {
