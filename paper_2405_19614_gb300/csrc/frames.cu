@@ -9,36 +9,68 @@
 
 namespace gs {
 
-// Four pixels a thread: 12 colour bytes (three 4-byte words) and four depth
-// values (one 8-byte word) in, three float4 of colour and one of depth out.
-__global__ void __launch_bounds__(256) decode_kernel(const uint32_t *__restrict__ rgb8w,
-                                                     const uint2 *__restrict__ depth16w, int64_t n_quads,
-                                                     float depth_scale, float4 *__restrict__ rgb,
-                                                     float4 *__restrict__ depth)
+constexpr int kDecodeThreads = 256;
+constexpr int kDecodeItems = 4;   // in flight a thread (two or eight: 27.5, 29.0 us)
+constexpr int kDecodeBlocks = 8;  // an SM
+
+// c / 255 correctly rounded, for whole c in [0, 255]: the product with the
+// rounded reciprocal, corrected by its exact remainder (Markstein 1990); equal
+// to the quotient's nearest FP32 number for all 256 values.
+__device__ __forceinline__ float over_255(uint32_t c)
 {
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n_quads;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t w[3] = {rgb8w[3 * q], rgb8w[3 * q + 1], rgb8w[3 * q + 2]};
-        float c[12];
-        #pragma unroll
-        for (int k = 0; k < 12; k++) c[k] = __fdiv_rn((float)((w[k >> 2] >> (8 * (k & 3))) & 0xffu), 255.0f);
-        rgb[3 * q] = make_float4(c[0], c[1], c[2], c[3]);
-        rgb[3 * q + 1] = make_float4(c[4], c[5], c[6], c[7]);
-        rgb[3 * q + 2] = make_float4(c[8], c[9], c[10], c[11]);
-        const uint2 d = depth16w[q];
-        depth[q] = make_float4(__fmul_rn((float)(d.x & 0xffffu), depth_scale), __fmul_rn((float)(d.x >> 16), depth_scale),
-                               __fmul_rn((float)(d.y & 0xffffu), depth_scale), __fmul_rn((float)(d.y >> 16), depth_scale));
-    }
+    constexpr float r = 1.0f / 255.0f;
+    const float x = (float)c, q = __fmul_rn(x, r);
+    return __fmaf_rn(__fmaf_rn(-255.0f, q, x), r, q);
 }
 
-// The last n mod 4 pixels, one a thread.
-__global__ void decode_tail_kernel(const uint8_t *__restrict__ rgb8, const uint16_t *__restrict__ depth16, int64_t p0,
-                                   int64_t n, float depth_scale, float *__restrict__ rgb, float *__restrict__ depth)
+// A frame is two flat arrays: output float4 k of the colours holds the four
+// bytes of input word k, whatever pixels they belong to, and output float4 k of
+// the depths the four values of input word pair k.  Items are the colour words,
+// then the depth word pairs; consecutive threads take consecutive items, so
+// every load and store of a warp is one contiguous span.  Bound: HBM.  Four
+// pixels a thread, each float4 stored 48 bytes from its neighbour's and twelve
+// divisions: 29.0 us for eight 1200x680 frames (28.0 with the stores in order),
+// now 24.8 us, 137 MB at 5.5 TB/s.  The last bytes and values beyond whole words
+// go one a thread of block 0 (they were a launch of their own).
+__global__ void __launch_bounds__(kDecodeThreads) decode_kernel(const uint8_t *__restrict__ rgb8,
+                                                                const uint16_t *__restrict__ depth16, int64_t n_pixels,
+                                                                float depth_scale, float *__restrict__ rgb,
+                                                                float *__restrict__ depth)
 {
-    const int64_t p = p0 + threadIdx.x;
-    if (p >= n) return;
-    for (int ch = 0; ch < 3; ch++) rgb[3 * p + ch] = __fdiv_rn((float)rgb8[3 * p + ch], 255.0f);
-    depth[p] = __fmul_rn((float)depth16[p], depth_scale);
+    const uint32_t *cw = reinterpret_cast<const uint32_t *>(rgb8);
+    const uint2 *dw = reinterpret_cast<const uint2 *>(depth16);
+    float4 *co = reinterpret_cast<float4 *>(rgb), *po = reinterpret_cast<float4 *>(depth);
+    const int64_t colours = 3 * n_pixels / 4, items = colours + n_pixels / 4;
+    const int64_t stride = (int64_t)gridDim.x * kDecodeThreads;
+    for (int64_t i0 = (int64_t)blockIdx.x * kDecodeThreads + threadIdx.x; i0 < items; i0 += kDecodeItems * stride) {
+        uint2 w[kDecodeItems];
+        #pragma unroll
+        for (int k = 0; k < kDecodeItems; k++) {
+            const int64_t i = i0 + k * stride;
+            w[k] = make_uint2(0u, 0u);
+            if (i < colours) w[k].x = __ldcs(cw + i);
+            else if (i < items) w[k] = __ldcs(dw + (i - colours));
+        }
+        #pragma unroll
+        for (int k = 0; k < kDecodeItems; k++) {
+            const int64_t i = i0 + k * stride;
+            if (i < colours) {
+                const uint32_t c = w[k].x;
+                __stcs(co + i, make_float4(over_255(c & 0xffu), over_255((c >> 8) & 0xffu),
+                                           over_255((c >> 16) & 0xffu), over_255(c >> 24)));
+            } else if (i < items) {
+                const uint2 d = w[k];
+                __stcs(po + (i - colours),
+                       make_float4(__fmul_rn((float)(d.x & 0xffffu), depth_scale), __fmul_rn((float)(d.x >> 16), depth_scale),
+                                   __fmul_rn((float)(d.y & 0xffffu), depth_scale), __fmul_rn((float)(d.y >> 16), depth_scale)));
+            }
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 4) {
+        const int64_t c = 4 * colours + threadIdx.x, d = n_pixels / 4 * 4 + threadIdx.x;
+        if (c < 3 * n_pixels) rgb[c] = over_255(rgb8[c]);
+        if (d < n_pixels) depth[d] = __fmul_rn((float)depth16[d], depth_scale);
+    }
 }
 
 }  // namespace gs
@@ -55,15 +87,9 @@ extern "C" gs_status_t gs_decode_keyframes(const uint8_t *rgb8, const uint16_t *
         (reinterpret_cast<uintptr_t>(rgb) & 15) || (reinterpret_cast<uintptr_t>(depth) & 15))
         return GS_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    const int64_t quads = n_pixels / 4;
-    if (quads > 0) {
-        int64_t blocks = (quads + 255) / 256;
-        const int64_t cap = (int64_t)num_sms() * 8;
-        if (blocks > cap) blocks = cap;
-        decode_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const uint32_t *>(rgb8),
-                                                        reinterpret_cast<const uint2 *>(depth16), quads, depth_scale,
-                                                        reinterpret_cast<float4 *>(rgb), reinterpret_cast<float4 *>(depth));
-    }
-    if (4 * quads < n_pixels) decode_tail_kernel<<<1, 4, 0, s>>>(rgb8, depth16, 4 * quads, n_pixels, depth_scale, rgb, depth);
+    int64_t blocks = (n_pixels + kDecodeThreads - 1) / kDecodeThreads;
+    const int64_t cap = (int64_t)num_sms() * kDecodeBlocks;
+    if (blocks > cap) blocks = cap;
+    decode_kernel<<<(unsigned)blocks, kDecodeThreads, 0, s>>>(rgb8, depth16, n_pixels, depth_scale, rgb, depth);
     return launch_status();
 }
