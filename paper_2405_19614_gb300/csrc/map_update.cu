@@ -12,6 +12,7 @@
 // kept.
 // Both selections are compactions done with a per-block scan, so the order of
 // new and surviving Gaussians is deterministic (pixel order; index order).
+#include "chain.cuh"
 #include "common.cuh"
 
 namespace gs {
@@ -45,6 +46,7 @@ __device__ __forceinline__ uint32_t block_scan_u32(uint32_t x, uint32_t *tmp, ui
 template <typename SEL>
 __global__ void __launch_bounds__(kSelThreads) select_count_kernel(SEL sel, int64_t n, uint32_t *counts)
 {
+    chain_go();
     __shared__ uint32_t tmp[kSelThreads / 32];
     const int64_t first = (int64_t)blockIdx.x * kSelChunk + (int64_t)threadIdx.x * kSelItems;
     uint32_t c = 0;
@@ -60,6 +62,8 @@ __global__ void __launch_bounds__(kSelThreads) select_count_kernel(SEL sel, int6
 __global__ void __launch_bounds__(1024) select_scan_kernel(uint32_t *counts, int64_t nb, uint32_t *total,
                                                            uint32_t capacity_left, uint32_t *stored, uint32_t *status)
 {
+    chain_go();
+    chain_wait();
     __shared__ uint32_t tmp[32];
     __shared__ uint32_t carry;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -119,6 +123,8 @@ constexpr uint32_t kDensifySplit = 4;
 // (57 us with one block a chunk and a division and a load in the SH loop).
 __global__ void __launch_bounds__(kSelThreads) densify_write_kernel(DensifyArgs a, ViewTable vt, const uint32_t *offsets)
 {
+    chain_go();
+    chain_wait();
     __shared__ uint32_t tmp[kSelThreads / 32];
     __shared__ float s_mean[3 * kSelChunk];
     __shared__ float s_ls[kSelChunk];
@@ -195,6 +201,8 @@ struct PruneSel {
 __global__ void __launch_bounds__(kSelThreads) prune_index_kernel(const float *opacity_logit, int64_t n, float min_logit,
                                                                    const uint32_t *offsets, int32_t *new_index)
 {
+    chain_go();
+    chain_wait();
     __shared__ uint32_t tmp[kSelThreads / 32];
     const int64_t first = (int64_t)blockIdx.x * kSelChunk + (int64_t)threadIdx.x * kSelItems;
     bool keep[kSelItems];
@@ -311,7 +319,7 @@ extern "C" gs_status_t gs_densify(const float *alpha, const float *target_rgb, c
     DensifySel sel{alpha, target_depth, threshold};
     select_count_kernel<<<(unsigned)nb, kSelThreads, 0, s>>>(sel, P, counts);
     uint32_t *total = counts + nb;
-    select_scan_kernel<<<1, 1024, 0, s>>>(counts, nb, total, (uint32_t)left, n_added, status);
+    launch_chained(select_scan_kernel, 1, 1024, 0, s, counts, nb, total, (uint32_t)left, n_added, status);
     DensifyArgs a;
     a.alpha = alpha;
     a.depth = target_depth;
@@ -328,7 +336,7 @@ extern "C" gs_status_t gs_densify(const float *alpha, const float *target_rgb, c
     a.n_old = n_old;
     a.capacity = capacity;
     a.P = P;
-    densify_write_kernel<<<dim3((unsigned)nb, kDensifySplit), kSelThreads, 0, s>>>(a, vt, counts);
+    launch_chained(densify_write_kernel, dim3((unsigned)nb, kDensifySplit), kSelThreads, 0, s, a, vt, counts);
     return launch_status();
 }
 
@@ -347,8 +355,8 @@ extern "C" gs_status_t gs_prune_select(const float *opacity_logit, int64_t n, fl
     const int64_t nb = (n + kSelChunk - 1) / kSelChunk;
     PruneSel sel{opacity_logit, min_logit};
     select_count_kernel<<<(unsigned)nb, kSelThreads, 0, s>>>(sel, n, counts);
-    select_scan_kernel<<<1, 1024, 0, s>>>(counts, nb, n_kept, 0xffffffffu, nullptr, nullptr);
-    prune_index_kernel<<<(unsigned)nb, kSelThreads, 0, s>>>(opacity_logit, n, min_logit, counts, new_index);
+    launch_chained(select_scan_kernel, 1, 1024, 0, s, counts, nb, n_kept, 0xffffffffu, nullptr, nullptr);
+    launch_chained(prune_index_kernel, (unsigned)nb, kSelThreads, 0, s, opacity_logit, n, min_logit, counts, new_index);
     return launch_status();
 }
 

@@ -21,6 +21,7 @@
 // and clears the 2D gradient entries it consumed.  Keeping the SH state out of
 // the geometry kernel keeps it at a register count that lets many warps hide
 // latency.
+#include "chain.cuh"
 #include "common.cuh"
 #include "async_copy.cuh"
 #include "sh.cuh"
@@ -209,6 +210,7 @@ constexpr int kColorThreads = 32 * kPbwdWarps;
 template <int DEG>
 __global__ void __launch_bounds__(kColorThreads, 3) project_bwd_color_kernel(ProjectBwdArgs a, ViewTable vt)
 {
+    chain_go();
     using T = ShTile<DEG>;
     constexpr int K = T::K;
     __shared__ float s_E[GS_MAX_VIEWS][12];
@@ -373,6 +375,8 @@ __global__ void __launch_bounds__(kColorThreads, 3) project_bwd_color_kernel(Pro
 // warps hide more of them than the spill costs.
 __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(ProjectBwdArgs a, ViewTable vt)
 {
+    chain_go();
+    chain_wait();
     __shared__ float s_E[GS_MAX_VIEWS][12];
     __shared__ float s_tw[GS_MAX_VIEWS][6];
     __shared__ __align__(16) float s_twt[kPbwdWarps][kTwGroup * 6][kTwPitch];
@@ -656,7 +660,7 @@ extern "C" gs_status_t gs_project_bwd(const gs_params_t *params, const gs_view_t
     default: project_bwd_color_kernel<3><<<cblocks, kColorThreads, 0, s>>>(a, vt); break;
     }
     const unsigned gblocks = (unsigned)((params->n + threads - 1) / threads);
-    project_bwd_geom_kernel<<<gblocks, threads, 0, s>>>(a, vt);
+    launch_chained(project_bwd_geom_kernel, gblocks, threads, 0, s, a, vt);
     return launch_status();
 }
 

@@ -33,6 +33,7 @@
 // and keeps the 16 input rows it needs in registers.
 #include <mutex>
 
+#include "chain.cuh"
 #include "common.cuh"
 #include "async_copy.cuh"
 #include "tma.cuh"
@@ -201,6 +202,7 @@ __global__ void __launch_bounds__(kSsimThreads) ssim_stats_kernel(const float *_
                                                                   float *__restrict__ partial, float *loss,
                                                                   float scale, float constant)
 {
+    chain_go();
     extern __shared__ float smem[];
     float *s_in = smem;                                   // [2][rows][127]: x, y halo, RGB interleaved
     float *s_h = smem + 2 * kSsimRows * kSsimInPitchXY;  // [4][rows][33]
@@ -310,6 +312,8 @@ __global__ void __launch_bounds__(kSsimThreads) ssim_grad_kernel(const float *__
                                                                  const float *__restrict__ partial,
                                                                  float *__restrict__ d_rgb, float gsc)
 {
+    chain_go();
+    chain_wait();
     extern __shared__ float smem[];
     constexpr int kBuf = 3 * kSsimRows * kSsimInPitch;
     float *s_in = smem;                                 // [2][3][rows][43]: a channel's three maps, double-buffered
@@ -429,6 +433,8 @@ __global__ void __launch_bounds__(kSsimThreads, GS_SSIM_GRAD_TMA_BLOCKS) ssim_gr
                                                                      float *__restrict__ d_rgb, float gsc,
                                                                      uint32_t *status, uint32_t extra_tx)
 {
+    chain_go();
+    chain_wait();
     extern __shared__ __align__(128) float smem[];
     float *s_in = smem;                                 // [3][rows][52]: a channel's three maps (TMA box)
     float *s_h = smem + 3 * kSsimRows * kSsimTmaPitch;  // [3][rows][33]
@@ -674,10 +680,10 @@ static gs_status_t ssim_launch(const float *rgb, const float *target_rgb, const 
     std::lock_guard<std::mutex> lock(maps_mu);
     // (the timeout check stays with the views whose rows need no padding)
     if ((extra_tx == 0 || rows_aligned(T)) && make_ssim_maps(T, partial, &maps))
-        ssim_grad_tma_kernel<<<blocks, kSsimThreads, kSsimGradTmaSmem, s>>>(rgb, target_rgb, T, maps, d_rgb, scale,
-                                                                            status, extra_tx);
+        launch_chained(ssim_grad_tma_kernel, blocks, kSsimThreads, kSsimGradTmaSmem, s, rgb, target_rgb, T, maps, d_rgb,
+                       scale, status, extra_tx);
     else if (extra_tx == 0)
-        ssim_grad_kernel<<<blocks, kSsimThreads, kSsimGradSmem, s>>>(rgb, target_rgb, T, partial, d_rgb, scale);
+        launch_chained(ssim_grad_kernel, blocks, kSsimThreads, kSsimGradSmem, s, rgb, target_rgb, T, partial, d_rgb, scale);
     else
         return GS_ERR_UNSUPPORTED;
     return launch_status();

@@ -26,6 +26,7 @@
 //   1M, 8 views of 1200x680 (32x16 tiles), 4.0M   235 against 305 us
 //   4M, 16 views (lists up to 59,000), 28.2M      1.67 against 2.36 ms
 #include "binning.cuh"
+#include "chain.cuh"
 #include "common.cuh"
 
 namespace gs {
@@ -315,6 +316,8 @@ __device__ __noinline__ void cut_to_capacity(const ListArgs &a, const ViewTable 
 
 __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(ListArgs a, ViewTable vt, bool advance)
 {
+    chain_go();
+    chain_wait();
     const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
     if (threadIdx.x == 0) *a.state = ListState{};
     const uint64_t pairs = scan_tiles(a, n_tiles, advance);
@@ -339,6 +342,7 @@ __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(ListArgs a, Vie
 template <bool PRIVATE>
 __global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_count_kernel(ListArgs a, ViewTable vt, uint32_t blocks_per_view)
 {
+    chain_go();
     extern __shared__ __align__(16) unsigned char s_raw[];
     uint32_t *s_tile = reinterpret_cast<uint32_t *>(s_raw);  // the view's tiles
     const uint32_t v = blockIdx.x / blocks_per_view, b = blockIdx.x - v * blocks_per_view;
@@ -384,6 +388,8 @@ __global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_count_kernel(
 template <bool PRIVATE>
 __global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_scatter_kernel(ListArgs a, ViewTable vt, uint32_t blocks_per_view)
 {
+    chain_go();
+    chain_wait();
     extern __shared__ __align__(16) unsigned char s_raw[];
     uint32_t *s_tile = reinterpret_cast<uint32_t *>(s_raw);
     const uint32_t v = blockIdx.x / blocks_per_view, b = blockIdx.x - v * blocks_per_view;
@@ -495,6 +501,8 @@ __device__ __forceinline__ void group_sort(const unsigned long long *src, uint32
 // one chunk is finished here; the chunks of longer ones go back sorted.
 __global__ void __launch_bounds__(kSortBlock, 2) tile_sort_kernel(ListArgs a, uint32_t n_tiles, uint32_t extra)
 {
+    chain_go();
+    chain_wait();
     extern __shared__ __align__(16) unsigned char s_raw[];
     unsigned long long *s = reinterpret_cast<unsigned long long *>(s_raw);
     if (blockIdx.x < extra) {
@@ -545,6 +553,8 @@ __global__ void __launch_bounds__(kSortBlock, 2) tile_sort_kernel(ListArgs a, ui
 // own chunk plus the words below it in the tile's other chunks.
 __global__ void __launch_bounds__(kMergeThreads) tile_merge_kernel(ListArgs a)
 {
+    chain_go();
+    chain_wait();
     const uint32_t n_long = a.state->n_long;
     for (uint32_t j = blockIdx.x; j < n_long; j += gridDim.x) {
         const uint2 tc = a.long_chunks[j];
@@ -586,8 +596,8 @@ static gs_status_t launch_walks(const ListArgs &a, const ViewTable &vt, uint32_t
             return GS_ERR_CUDA;
     }
     tile_count_kernel<PRIVATE><<<grid, kListThreads, smem, s>>>(a, vt, blocks_per_view);
-    tile_scan_kernel<<<1, kScanThreads, 0, s>>>(a, vt, !PRIVATE);
-    tile_scatter_kernel<PRIVATE><<<grid, kListThreads, smem, s>>>(a, vt, blocks_per_view);
+    launch_chained(tile_scan_kernel, 1, kScanThreads, 0, s, a, vt, !PRIVATE);
+    launch_chained(tile_scatter_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
     return launch_status();
 }
 
@@ -656,8 +666,8 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     if (cudaFuncSetAttribute(tile_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem) != cudaSuccess)
         return GS_ERR_CUDA;
     const unsigned groups = kSortBlock / kSortGroup;
-    tile_sort_kernel<<<(n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s>>>(a, n_tiles, extra);
-    tile_merge_kernel<<<(unsigned)num_sms() * 8, kMergeThreads, 0, s>>>(a);
+    launch_chained(tile_sort_kernel, (n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s, a, n_tiles, extra);
+    launch_chained(tile_merge_kernel, (unsigned)num_sms() * 8, kMergeThreads, 0, s, a);
     return launch_status();
 }
 
