@@ -120,15 +120,56 @@ __device__ __forceinline__ bool world_covariance(const float ls[3], const float 
     return true;
 }
 
+// A quick test that a Gaussian in front of the camera touches no tile, ahead of
+// the covariance and the radius: about half of the Gaussians of a room are in
+// front of a camera and half of those beside its image.  The 2D covariance is
+// J W S W^T J^T + blur I, and with the infinity norms of S, W W^T and J J^T
+// (each at least the spectral norm)
+//   lambda_max <= |S| |W W^T| F / z^2 + blur,
+//   F = max(fx^2 (1 + lx^2), fy^2 (1 + ly^2)) + fx fy lx ly
+// (|x/z| and |y/z| are clamped to lx and ly in J), so the radius is at most
+// 3 (sqrt(|S|) sqrt(|W W^T| F) / |z| + sqrt(blur)) + 1.  The bound is taken a
+// thousandth and a pixel larger, far above the rounding of both sides, and the
+// mean from an approximate reciprocal within 1e-5 of its terms; whatever is not
+// finite fails the comparisons and goes on to the contract.  reach: the view's
+// 3.003 sqrt(|W W^T| F) and 3.003 sqrt(blur) + 2.  (4M Gaussians, 16 views:
+// 766 -> 725 us for the kernel; 1M, 8 views: 100 -> 90.)
+__device__ __forceinline__ bool beside_the_image(float x, float y, float z, float root_s, const float *reach,
+                                                 const ViewInfo &V)
+{
+    const float rz = __fdividef(1.0f, z);
+    const float r = fmaf(reach[0] * root_s, fabsf(rz), reach[1]);
+    const float px = V.fx * x * rz, py = V.fy * y * rz;
+    const float ru = fmaf(1e-5f, fabsf(px) + fabsf(V.cx), r), rv = fmaf(1e-5f, fabsf(py) + fabsf(V.cy), r);
+    const float u = px + V.cx, v = py + V.cy;
+    return u + ru < 0.0f || v + rv < 0.0f || u - ru > (float)(V.tiles_x * V.tile_w) ||
+           v - rv > (float)(V.tiles_y * V.tile_h);
+}
+
+// Largest absolute row sum (the infinity norm) of a 3 x 3 matrix.
+__device__ __forceinline__ float norm_inf(const float A[3][3])
+{
+    float n = 0.0f;
+    #pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const float r = fabsf(A[i][0]) + fabsf(A[i][1]) + fabsf(A[i][2]);
+        n = r > n || !(r == r) ? r : n;  // a NaN stays
+    }
+    return n;
+}
+
 // The per-view part.  Returns false when the Gaussian touches no tile.  lim:
-// the view's (limx, limy) = 1.3 (0.5 width / fx, 0.5 height / fy).
-__device__ __forceinline__ bool geometry(const float m[3], const float S[3][3], const float *E, const ViewInfo &V,
-                                         const float *lim, float near_z, float blur, Geom &g)
+// the view's (limx, limy) = 1.3 (0.5 width / fx, 0.5 height / fy); root_s and
+// reach as in beside_the_image.
+__device__ __forceinline__ bool geometry(const float m[3], const float S[3][3], float root_s, const float *E,
+                                         const ViewInfo &V, const float *lim, const float *reach, float near_z,
+                                         float blur, Geom &g)
 {
     float x = ADD(ADD(ADD(MUL(E[0], m[0]), MUL(E[1], m[1])), MUL(E[2], m[2])), E[3]);
     float y = ADD(ADD(ADD(MUL(E[4], m[0]), MUL(E[5], m[1])), MUL(E[6], m[2])), E[7]);
     float z = ADD(ADD(ADD(MUL(E[8], m[0]), MUL(E[9], m[1])), MUL(E[10], m[2])), E[11]);
     if (!(z > near_z)) return false;
+    if (beside_the_image(x, y, z, root_s, reach, V)) return false;
 
     const float limx = lim[0], limy = lim[1];
     float xz = DIV(x, z), yz = DIV(y, z);
@@ -334,6 +375,7 @@ __global__ void __launch_bounds__(128) project_kernel(ProjectArgs a, ViewTable v
     __shared__ float s_E[GS_MAX_VIEWS][12];
     __shared__ float s_c[GS_MAX_VIEWS][3];
     __shared__ float s_lim[GS_MAX_VIEWS][2];
+    __shared__ float s_reach[GS_MAX_VIEWS][2];
     for (int k = threadIdx.x; k < vt.n_views * 12; k += blockDim.x) s_E[k / 12][k % 12] = a.viewmats[k];
     __syncthreads();
     for (int v = threadIdx.x; v < vt.n_views; v += blockDim.x) {
@@ -345,6 +387,16 @@ __global__ void __launch_bounds__(128) project_kernel(ProjectArgs a, ViewTable v
         const ViewInfo &V = vt.v[v];
         s_lim[v][0] = __fmul_rn(1.3f, __fdiv_rn(__fmul_rn(0.5f, (float)V.width), V.fx));
         s_lim[v][1] = __fmul_rn(1.3f, __fdiv_rn(__fmul_rn(0.5f, (float)V.height), V.fy));
+        float WW[3][3];
+        #pragma unroll
+        for (int i = 0; i < 3; i++)
+            #pragma unroll
+            for (int j = 0; j < 3; j++)
+                WW[i][j] = E[4 * i] * E[4 * j] + E[4 * i + 1] * E[4 * j + 1] + E[4 * i + 2] * E[4 * j + 2];
+        const float lx = s_lim[v][0], ly = s_lim[v][1];
+        const float F = fmaxf(V.fx * V.fx * (1.0f + lx * lx), V.fy * V.fy * (1.0f + ly * ly)) + V.fx * V.fy * lx * ly;
+        s_reach[v][0] = 3.003f * sqrtf(norm_inf(WW) * F);
+        s_reach[v][1] = 3.003f * sqrtf(fmaxf(a.blur, 0.0f)) + 2.0f;
     }
     __syncthreads();
 
@@ -364,6 +416,7 @@ __global__ void __launch_bounds__(128) project_kernel(ProjectArgs a, ViewTable v
     const float log2o = geom_log2_opacity(__ldg(a.opacity_logit + i));
     float S[3][3];
     const bool cov_ok = world_covariance(ls, q, S);
+    const float root_s = cov_ok ? sqrtf(norm_inf(S)) : 0.0f;
     // the SH coefficients are read only for the views the Gaussian is drawn
     // in (they come from L1 after the first): 48 registers fewer a thread than
     // holding them across the view loop, and no read for a Gaussian no view draws
@@ -389,7 +442,7 @@ __global__ void __launch_bounds__(128) project_kernel(ProjectArgs a, ViewTable v
     for (int v = 0; v < vt.n_views; v++) {
         const int64_t o = (int64_t)v * a.n + i;
         Geom g;
-        if (!cov_ok || !geometry(m, S, s_E[v], vt.v[v], s_lim[v], a.near_z, a.blur, g)) {
+        if (!cov_ok || !geometry(m, S, root_s, s_E[v], vt.v[v], s_lim[v], s_reach[v], a.near_z, a.blur, g)) {
             a.radii[o] = 0;
             a.tiles_touched[o] = 0;
             continue;
