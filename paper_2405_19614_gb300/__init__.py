@@ -38,12 +38,15 @@ def _ptr(t):
         raise GsError("tensor must be on the GPU")
     if not t.is_contiguous():
         raise GsError("tensor must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    # the raw handle: the Stream object that torch.cuda.current_stream() makes
+    # around it took 3.0 us a call, of which a tracking step makes seven
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def make_views(intr, size, tile=None):

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "gs.h"
 
 namespace gs {
@@ -102,12 +104,46 @@ inline gs_status_t launch_status()
 
 inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 
+// A number per device that never changes, asked of the runtime once: get(dev)
+// on the first use on each of the first 64 devices, every time beyond.  (Two
+// threads may both ask; they get the same number.)
+struct PerDevice {
+    std::atomic<int> known[64] = {};
+    template <typename GET>
+    int operator()(GET get)
+    {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev < 0 || dev >= 64) return get(dev);
+        int x = known[dev].load(std::memory_order_relaxed);
+        if (x <= 0) {
+            x = get(dev);
+            known[dev].store(x, std::memory_order_relaxed);
+        }
+        return x;
+    }
+};
+
 inline int num_sms()
 {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
+    static PerDevice sms;
+    return sms([](int dev) {
+        int n = 0;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return n > 0 ? n : 1;
+    });
+}
+
+// Resident blocks per SM of a kernel without dynamic shared memory (the query
+// takes a microsecond or two a launch).
+template <typename K>
+inline int blocks_per_sm(PerDevice &known, K kernel, int threads)
+{
+    return known([&](int) {
+        int n = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, 0);
+        return n > 0 ? n : 1;
+    });
 }
 
 // Warp-wide sum.

@@ -468,9 +468,8 @@ static gs_status_t launch_fwd(RenderFwdArgs a, ViewTable vt, const CUtensorMap &
     // work items: the bands of every tile of every view (tile shapes are per view)
     a.n_items = render_items(&vt, BW, PPT * (32 / BW));
     auto kern = render_fwd_kernel<PPT, BW, CH, TMA, STATS, LOSS, ASYNC>;
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kRenderThreads, 0);
-    const int64_t slots = (int64_t)num_sms() * (per_sm > 0 ? per_sm : 1);
+    static PerDevice per_sm;
+    const int64_t slots = (int64_t)num_sms() * blocks_per_sm(per_sm, kern, kRenderThreads);
     const int64_t blocks_needed = ((int64_t)a.n_items + kRenderThreads / 32 - 1) / (kRenderThreads / 32);
     const int grid = (int)(slots < blocks_needed ? slots : blocks_needed);
     // every item has a warp of its own when the grid holds them all: no counter

@@ -663,8 +663,14 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     if (st != GS_OK) return st;
     const uint32_t extra = (uint32_t)num_sms() * 2;
     const size_t sort_smem = sizeof(unsigned long long) * kTileChunk;
-    if (cudaFuncSetAttribute(tile_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem) != cudaSuccess)
-        return GS_ERR_CUDA;
+    static PerDevice allowed;  // 1 once the device has been told of the kernel's shared memory
+    const int ok = allowed([&](int) {
+        return cudaFuncSetAttribute(tile_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem) ==
+                       cudaSuccess
+                   ? 1
+                   : 0;
+    });
+    if (!ok) return GS_ERR_CUDA;
     const unsigned groups = kSortBlock / kSortGroup;
     launch_chained(tile_sort_kernel, (n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s, a, n_tiles, extra);
     launch_chained(tile_merge_kernel, (unsigned)num_sms() * 8, kMergeThreads, 0, s, a);
