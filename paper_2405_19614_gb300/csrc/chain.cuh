@@ -20,26 +20,56 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace gs {
 
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A launch with its attributes: chained (or not), in clusters of `cluster` blocks.
 template <typename... P, typename... A>
-inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+inline void launch_with(bool chained, int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                        cudaStream_t s, A... args)
 {
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2] = {};
     cudaLaunchConfig_t cfg = {};
+    if (chained) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // errors are read by launch_status
+}
+
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    launch_with(true, 1, kernel, grid, block, smem, s, args...);
+}
+
+// Clears n words for the kernel chained after it (a memset would end before that
+// kernel's launch begins).
+static __global__ void chain_clear_kernel(uint32_t *p, uint32_t n)
+{
+    chain_go();
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0u;
+}
+
+inline void launch_clear(uint32_t *p, uint32_t n, cudaStream_t s)
+{
+    const unsigned blocks = (n + 1023) / 1024;
+    chain_clear_kernel<<<blocks < 512 ? blocks : 512, n < 256 ? 32 : 256, 0, s>>>(p, n);
 }
 
 }  // namespace gs

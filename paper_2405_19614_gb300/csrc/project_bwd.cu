@@ -211,6 +211,7 @@ template <int DEG>
 __global__ void __launch_bounds__(kColorThreads, 3) project_bwd_color_kernel(ProjectBwdArgs a, ViewTable vt)
 {
     chain_go();
+    chain_wait();
     using T = ShTile<DEG>;
     constexpr int K = T::K;
     __shared__ float s_E[GS_MAX_VIEWS][12];
@@ -612,9 +613,10 @@ __global__ void __launch_bounds__(128, 5) project_bwd_geom_kernel(ProjectBwdArgs
 
 using namespace gs;
 
-extern "C" gs_status_t gs_project_bwd(const gs_params_t *params, const gs_view_t *views, const float *viewmats,
-                                      int32_t n_views, const gs_options_t *opt, const gs_projected_t *proj,
-                                      float *grad2d, gs_param_grads_t *grads, float *d_twist, void *stream)
+// chained: the launch before on the stream is the compositing's backward of the same call.
+static gs_status_t project_bwd(const gs_params_t *params, const gs_view_t *views, const float *viewmats,
+                               int32_t n_views, const gs_options_t *opt, const gs_projected_t *proj, float *grad2d,
+                               gs_param_grads_t *grads, float *d_twist, bool chained, void *stream)
 {
     if (!params || !viewmats || !opt || !proj || !grad2d) return GS_ERR_INVALID_ARG;
     if (!grads && !d_twist) return GS_ERR_INVALID_ARG;
@@ -654,14 +656,21 @@ extern "C" gs_status_t gs_project_bwd(const gs_params_t *params, const gs_view_t
     // colour first: the geometry kernel clears the 2D gradients after use
     const unsigned cblocks = (unsigned)((params->n + kColorThreads - 1) / kColorThreads);
     switch (params->sh_degree) {
-    case 0: project_bwd_color_kernel<0><<<cblocks, kColorThreads, 0, s>>>(a, vt); break;
-    case 1: project_bwd_color_kernel<1><<<cblocks, kColorThreads, 0, s>>>(a, vt); break;
-    case 2: project_bwd_color_kernel<2><<<cblocks, kColorThreads, 0, s>>>(a, vt); break;
-    default: project_bwd_color_kernel<3><<<cblocks, kColorThreads, 0, s>>>(a, vt); break;
+    case 0: launch_with(chained, 1, project_bwd_color_kernel<0>, cblocks, kColorThreads, 0, s, a, vt); break;
+    case 1: launch_with(chained, 1, project_bwd_color_kernel<1>, cblocks, kColorThreads, 0, s, a, vt); break;
+    case 2: launch_with(chained, 1, project_bwd_color_kernel<2>, cblocks, kColorThreads, 0, s, a, vt); break;
+    default: launch_with(chained, 1, project_bwd_color_kernel<3>, cblocks, kColorThreads, 0, s, a, vt); break;
     }
     const unsigned gblocks = (unsigned)((params->n + threads - 1) / threads);
     launch_chained(project_bwd_geom_kernel, gblocks, threads, 0, s, a, vt);
     return launch_status();
+}
+
+extern "C" gs_status_t gs_project_bwd(const gs_params_t *params, const gs_view_t *views, const float *viewmats,
+                                      int32_t n_views, const gs_options_t *opt, const gs_projected_t *proj,
+                                      float *grad2d, gs_param_grads_t *grads, float *d_twist, void *stream)
+{
+    return project_bwd(params, views, viewmats, n_views, opt, proj, grad2d, grads, d_twist, false, stream);
 }
 
 extern "C" gs_status_t gs_render_bwd(const gs_params_t *params, const gs_view_t *views, const float *viewmats,
@@ -674,5 +683,5 @@ extern "C" gs_status_t gs_render_bwd(const gs_params_t *params, const gs_view_t 
     gs_status_t st = gs_render_bwd_splats(proj, params->n, bins, views, n_views, img, d_rgb, d_depth, d_alpha,
                                           grad2d, work_counter, stream);
     if (st != GS_OK) return st;
-    return gs_project_bwd(params, views, viewmats, n_views, opt, proj, grad2d, grads, d_twist, stream);
+    return project_bwd(params, views, viewmats, n_views, opt, proj, grad2d, grads, d_twist, true, stream);
 }

@@ -41,6 +41,7 @@
 #include <type_traits>
 
 #include "async_copy.cuh"
+#include "chain.cuh"
 #include "common.cuh"
 #include "render.cuh"
 #include "tma.cuh"
@@ -112,6 +113,8 @@ __global__ void __launch_bounds__(kRenderThreads, RenderOccupancy<PPT, TMA || AS
     render_bwd_kernel(RenderBwdArgs a, ViewTable vt, const __grid_constant__ CUtensorMap rec_map)
 {
     static_assert(!(TMA && ASYNC) && (!ASYNC || CH == 32), "one staging mode; asynchronous copies of 32 entries");
+    chain_go();  // the projection's backward, in a call of both
+    chain_wait();
     constexpr int WARPS = kRenderThreads / 32;
     constexpr int RS = 32 / BW;   // rows between a thread's pixels
     constexpr int BH = PPT * RS;  // band height (width BW)
@@ -571,9 +574,10 @@ static gs_status_t launch_bwd(RenderBwdArgs a, ViewTable vt, const CUtensorMap &
     const int grid = (int)(slots < blocks_needed ? slots : blocks_needed);
     // every item has a warp of its own when the grid holds them all: no counter
     // to clear and none to wait for (2 us less of a small image)
-    if (blocks_needed <= slots) a.work_counter = nullptr;
-    else if (cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
-    kern<<<grid > 0 ? grid : 1, kRenderThreads, 0, s>>>(a, vt, map);
+    const bool counted = blocks_needed > slots;
+    if (counted) launch_clear(a.work_counter, 1, s);
+    else a.work_counter = nullptr;
+    launch_with(counted, 1, kern, grid > 0 ? grid : 1, kRenderThreads, 0, s, a, vt, map);
     return launch_status();
 }
 

@@ -17,6 +17,7 @@
 // transmittance.  Warps never wait for one another.  The band shape and the
 // staging are chosen per workload by the autotuner.
 #include "async_copy.cuh"
+#include "chain.cuh"
 #include "common.cuh"
 #include "render.cuh"
 #include "tma.cuh"
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kRenderThreads, ASYNC ? RenderOccupancy<PPT, t
     RenderFwdArgs a, ViewTable vt, const __grid_constant__ CUtensorMap rec_map)
 {
     static_assert(!(TMA && ASYNC) && (!ASYNC || CH == 32), "one staging mode; asynchronous copies of 32 entries");
+    chain_wait();
     __shared__ float s_loss[kRenderThreads / 32];
     float lacc = 0.0f;  // LOSS: this thread's share of the loss
     constexpr int WARPS = kRenderThreads / 32;
@@ -474,24 +476,12 @@ static gs_status_t launch_fwd(RenderFwdArgs a, ViewTable vt, const CUtensorMap &
     const int grid = (int)(slots < blocks_needed ? slots : blocks_needed);
     // every item has a warp of its own when the grid holds them all: no counter
     // to clear and none to wait for (2 us less of a small image)
-    if (blocks_needed <= slots) a.work_counter = nullptr;
-    else if (cudaMemsetAsync(a.work_counter, 0, sizeof(uint32_t), s) != cudaSuccess) return GS_ERR_CUDA;
-    if constexpr (LOSS) {
-        a.loss_cluster = blocks_needed < kLossClusterTimes * slots ? kLossCluster : 1;
-        cudaLaunchAttribute attr = {};
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)a.loss_cluster;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = (unsigned)((grid + a.loss_cluster - 1) / a.loss_cluster * a.loss_cluster);
-        cfg.blockDim = kRenderThreads;
-        cfg.stream = s;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, kern, a, vt, map);
-    } else {
-        kern<<<grid > 0 ? grid : 1, kRenderThreads, 0, s>>>(a, vt, map);
-    }
+    const bool counted = blocks_needed > slots;
+    if (counted) launch_clear(a.work_counter, 1, s);
+    else a.work_counter = nullptr;
+    a.loss_cluster = LOSS && blocks_needed < kLossClusterTimes * slots ? kLossCluster : 1;
+    const int blocks = (grid > 0 ? grid + a.loss_cluster - 1 : a.loss_cluster) / a.loss_cluster * a.loss_cluster;
+    launch_with(counted, a.loss_cluster, kern, blocks, kRenderThreads, 0, s, a, vt, map);
     return launch_status();
 }
 

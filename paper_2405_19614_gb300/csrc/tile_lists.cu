@@ -353,6 +353,7 @@ __global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_count_kernel(
         for (uint32_t t = threadIdx.x; t < tiles; t += kListThreads) s_tile[t] = 0;
         __syncthreads();
     }
+    chain_wait();
     walk_view<false>(a, V, v, b * (kListThreads / 32) + threadIdx.x / 32, blocks_per_view * (kListThreads / 32),
                      PRIVATE ? CountPut{s_tile, 1u} : CountPut{&ranges[0].y, 2u});
     if (PRIVATE) {
@@ -595,7 +596,7 @@ static gs_status_t launch_walks(const ListArgs &a, const ViewTable &vt, uint32_t
             cudaFuncSetAttribute(tile_scatter_kernel<PRIVATE>, most, (int)smem) != cudaSuccess)
             return GS_ERR_CUDA;
     }
-    tile_count_kernel<PRIVATE><<<grid, kListThreads, smem, s>>>(a, vt, blocks_per_view);
+    launch_chained(tile_count_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
     launch_chained(tile_scan_kernel, 1, kScanThreads, 0, s, a, vt, !PRIVATE);
     launch_chained(tile_scatter_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
     return launch_status();
@@ -634,7 +635,7 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     a.keys = bins->keys;
     a.vals = bins->vals;
     const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
-    if (cudaMemsetAsync(a.ranges, 0, sizeof(uint2) * (size_t)n_tiles, s) != cudaSuccess) return GS_ERR_CUDA;
+    launch_clear(reinterpret_cast<uint32_t *>(a.ranges), 2 * n_tiles, s);
     uint32_t most_tiles = 0;
     for (int v = 0; v < vt.n_views; v++) {
         const uint32_t t = (uint32_t)(vt.v[v].tiles_x * vt.v[v].tiles_y);
@@ -673,7 +674,8 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     if (!ok) return GS_ERR_CUDA;
     const unsigned groups = kSortBlock / kSortGroup;
     launch_chained(tile_sort_kernel, (n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s, a, n_tiles, extra);
-    launch_chained(tile_merge_kernel, (unsigned)num_sms() * 8, kMergeThreads, 0, s, a);
+    // (no list is longer than a view has Gaussians)
+    if (n > kTileChunk) launch_chained(tile_merge_kernel, (unsigned)num_sms() * 8, kMergeThreads, 0, s, a);
     return launch_status();
 }
 

@@ -205,10 +205,10 @@ class MappingStep:
         self.v.copy_(news[2])
 
     def kernels_per_step(self):
-        """Kernels of this library launched by one run() (memsets excluded)."""
+        """Kernels of this library launched by one run() (clears excluded)."""
         r = self.rast
         if r.n * r.V <= 2048 * r.n_tiles and r.n_tiles <= 1 << 18:
-            k_bin = 5  # tile count, scan, scatter, sort, merge
+            k_bin = 4 + (r.n > 8192)  # tile count, scan, scatter, sort; the merge of long lists
         else:
             # record count, scan, compaction, 4 depth passes, pair count, scan, emission, the tile-id
             # passes (8 bits each) and the ranges
