@@ -259,6 +259,14 @@ gs_status_t gs_render_fwd(const gs_projected_t *proj, int64_t n, const gs_bins_t
                           const gs_view_t *views, int32_t n_views, gs_image_t *img,
                           uint32_t *work_counter, void *stream);
 
+/* gs_render_fwd that writes colour, depth and alpha a second time, into
+ * caller-owned arrays [P,3], [P], [P] (the outputs of a differentiable render,
+ * which outlive the image buffers), instead of three copies afterwards.
+ * Errors as gs_render_fwd, and GS_ERR_INVALID_ARG for null copies. */
+gs_status_t gs_render_fwd_copy(const gs_projected_t *proj, int64_t n, const gs_bins_t *bins, const gs_view_t *views,
+                               int32_t n_views, gs_image_t *img, float *copy_rgb, float *copy_depth,
+                               float *copy_alpha, uint32_t *work_counter, void *stream);
+
 /* a5 + a6 fused: gs_render_fwd that also evaluates gs_loss_l1 on each pixel as
  * it finishes (same arguments and results as gs_loss_l1 over all pixels of the
  * views: adds L to *loss, WRITES d_rgb [P,3] and d_depth [P]), so the image is

@@ -19,7 +19,7 @@ from . import _lib
 from ._lib import (GS_MAX_ADAM_GROUPS, GS_MAX_VIEWS, GS_TILE, GsAdamGroup, GsBins, GsError, GsImage, GsOptions,
                    GsParamGrads, GsParams, GsProjected, GsView, check)
 
-__all__ = ["gs_get_device_status", "gs_workspace_size", "gs_check_lookback_timeout", "gs_project", "gs_bin_sort", "gs_bin_sort_noalloc", "gs_render_fwd", "gs_render_fwd_l1", "gs_render_stats", "gs_set_render_variants",
+__all__ = ["gs_get_device_status", "gs_workspace_size", "gs_check_lookback_timeout", "gs_project", "gs_bin_sort", "gs_bin_sort_noalloc", "gs_render_fwd", "gs_render_fwd_copy", "gs_render_fwd_l1", "gs_render_stats", "gs_set_render_variants",
            "gs_get_render_variants", "gs_loss_l1", "gs_loss_ssim", "gs_check_ssim_timeout", "gs_render_bwd", "gs_render_bwd_splats",
            "gs_project_bwd", "gs_decode_keyframes", "gs_reproj_loss_grad", "gs_adam_step", "gs_pose_update", "gs_densify",
            "gs_prune_select", "gs_compact_rows", "gs_spatial_order_workspace_size", "gs_spatial_order",
@@ -156,6 +156,17 @@ def gs_bin_sort_noalloc(proj, n, views, bins, stream=None):
 def gs_render_fwd(proj, n, bins, views, img, work_counter, stream=None):
     check(lib().gs_render_fwd(ctypes.byref(_proj(proj)), n, ctypes.byref(_bins(bins)), views, len(views),
                               ctypes.byref(_img(img)), _ptr(work_counter), _stream(stream)), "gs_render_fwd")
+
+
+def gs_render_fwd_copy(proj, n, bins, views, img, copies, work_counter, stream=None):
+    """gs_render_fwd that also writes (rgb [P,3], depth [P], alpha [P]) into the tensors copies."""
+    rgb, depth, alpha = copies
+    P = img["depth"].numel()
+    if rgb.numel() != 3 * P or depth.numel() != P or alpha.numel() != P:
+        raise GsError("copy sizes disagree")
+    check(lib().gs_render_fwd_copy(ctypes.byref(_proj(proj)), n, ctypes.byref(_bins(bins)), views, len(views),
+                                   ctypes.byref(_img(img)), _ptr(rgb), _ptr(depth), _ptr(alpha), _ptr(work_counter),
+                                   _stream(stream)), "gs_render_fwd_copy")
 
 
 def gs_render_fwd_l1(proj, n, bins, views, img, work_counter, target_rgb, target_depth, w_c, w_d, use_gate, gamma,
@@ -376,11 +387,15 @@ class Rasterizer:
         self.work_counter = torch.zeros(1, dtype=i32, device=d)
         self.generation = 0
 
-    def forward(self, params, viewmats, stream=None):
-        """Project, bin and composite; results in self.img (device, async)."""
+    def forward(self, params, viewmats, stream=None, copies=None):
+        """Project, bin and composite; results in self.img (device, async) and,
+        when given, in the tensors copies = (rgb [P,3], depth [P], alpha [P])."""
         gs_project(params, self.views, viewmats, self.proj, self.near_z, self.blur, stream)
         gs_bin_sort(self.proj, self.n, self.views, self.bins, self.workspace, stream)
-        gs_render_fwd(self.proj, self.n, self.bins, self.views, self.img, self.work_counter, stream)
+        if copies is None:
+            gs_render_fwd(self.proj, self.n, self.bins, self.views, self.img, self.work_counter, stream)
+        else:
+            gs_render_fwd_copy(self.proj, self.n, self.bins, self.views, self.img, copies, self.work_counter, stream)
         self.generation += 1
         return self.img
 
@@ -426,13 +441,16 @@ class _RasterizeFn(torch.autograd.Function):
     def forward(ctx, rast, sh_degree, viewmats, twist, means, log_scales, quats, opacity_logit, sh):
         params = dict(means=means, log_scales=log_scales, quats=quats, opacity_logit=opacity_logit, sh=sh,
                       sh_degree=sh_degree)
-        img = rast.forward(params, viewmats)
+        # the outputs are written beside the rasterizer's images (three copies
+        # after the render took 21 us of launches)
+        out = [torch.empty_like(rast.img[k]) for k in ("rgb", "depth", "alpha")]
+        rast.forward(params, viewmats, copies=out)
         ctx.rast = rast
         ctx.generation = rast.generation
         ctx.sh_degree = sh_degree
         ctx.save_for_backward(viewmats, means, log_scales, quats, opacity_logit, sh)
         ctx.want_twist = twist is not None and twist.requires_grad
-        return img["rgb"].clone(), img["depth"].clone(), img["alpha"].clone()
+        return tuple(out)
 
     @staticmethod
     def backward(ctx, g_rgb, g_depth, g_alpha):

@@ -31,6 +31,7 @@ struct RenderFwdArgs {
     const uint32_t *ranges;
     float *rgb, *depth, *alpha, *final_T;
     uint32_t *n_contrib;
+    float *copy_rgb, *copy_depth, *copy_alpha;  // the images once more, or null
     uint32_t *n_eval, *n_blend;  // STATS variant only
     uint32_t *work_counter;  // null: the warps take the items in order, one each
     uint32_t *status;  // device error word (a bounded wait that expired), may be null
@@ -422,6 +423,13 @@ __global__ void __launch_bounds__(kRenderThreads, ASYNC ? RenderOccupancy<PPT, t
                 a.alpha[pix] = 1.0f - t;
                 a.final_T[pix] = t;
                 a.n_contrib[pix] = last[k];
+                if (!LOSS && a.copy_rgb) {
+                    a.copy_rgb[3 * pix + 0] = hi ? C0[i].y : C0[i].x;
+                    a.copy_rgb[3 * pix + 1] = hi ? C1[i].y : C1[i].x;
+                    a.copy_rgb[3 * pix + 2] = hi ? C2[i].y : C2[i].x;
+                    a.copy_depth[pix] = hi ? D[i].y : D[i].x;
+                    a.copy_alpha[pix] = 1.0f - t;
+                }
                 if (LOSS) {
                     // the a6 terms of this pixel, in the operations of gs_loss_l1
                     const float C[3] = {hi ? C0[i].y : C0[i].x, hi ? C1[i].y : C1[i].x, hi ? C2[i].y : C2[i].x};
@@ -527,9 +535,10 @@ static gs_status_t dispatch_fwd(int var, const RenderFwdArgs &a, const ViewTable
 
 using namespace gs;
 
-extern "C" gs_status_t gs_render_fwd(const gs_projected_t *proj, int64_t n, const gs_bins_t *bins,
-                                     const gs_view_t *views, int32_t n_views, gs_image_t *img,
-                                     uint32_t *work_counter, void *stream)
+// gs_render_fwd, with copies of the images (all three pointers, or none).
+static gs_status_t render_fwd(const gs_projected_t *proj, int64_t n, const gs_bins_t *bins, const gs_view_t *views,
+                              int32_t n_views, gs_image_t *img, float *copy_rgb, float *copy_depth, float *copy_alpha,
+                              uint32_t *work_counter, void *stream)
 {
     if (!proj || !bins || !img || !work_counter || n < 0) return GS_ERR_INVALID_ARG;
     ViewTable vt;
@@ -551,9 +560,27 @@ extern "C" gs_status_t gs_render_fwd(const gs_projected_t *proj, int64_t n, cons
     a.n_contrib = img->n_contrib;
     a.work_counter = work_counter;
     a.status = bins->status;
+    a.copy_rgb = copy_rgb;
+    a.copy_depth = copy_depth;
+    a.copy_alpha = copy_alpha;
     CUtensorMap map = {};
     const int var = prepare_fwd(a, vt, render_variant_fwd(vt.n_pix_total), &map);
     return dispatch_fwd<false>(var, a, vt, map, s);
+}
+
+extern "C" gs_status_t gs_render_fwd(const gs_projected_t *proj, int64_t n, const gs_bins_t *bins,
+                                     const gs_view_t *views, int32_t n_views, gs_image_t *img,
+                                     uint32_t *work_counter, void *stream)
+{
+    return render_fwd(proj, n, bins, views, n_views, img, nullptr, nullptr, nullptr, work_counter, stream);
+}
+
+extern "C" gs_status_t gs_render_fwd_copy(const gs_projected_t *proj, int64_t n, const gs_bins_t *bins,
+                                          const gs_view_t *views, int32_t n_views, gs_image_t *img, float *copy_rgb,
+                                          float *copy_depth, float *copy_alpha, uint32_t *work_counter, void *stream)
+{
+    if (!copy_rgb || !copy_depth || !copy_alpha) return GS_ERR_INVALID_ARG;
+    return render_fwd(proj, n, bins, views, n_views, img, copy_rgb, copy_depth, copy_alpha, work_counter, stream);
 }
 
 extern "C" gs_status_t gs_render_fwd_l1(const gs_projected_t *proj, int64_t n, const gs_bins_t *bins,
