@@ -146,6 +146,31 @@ inline int blocks_per_sm(PerDevice &known, K kernel, int threads)
     });
 }
 
+// A barrier of every thread of the cluster (whole warps).
+__device__ __forceinline__ void cluster_sync()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The block's rank in its cluster.
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// A float of this block's shared memory layout in block `rank` of the cluster.
+__device__ __forceinline__ float ld_cluster(const float *p, int rank)
+{
+    uint32_t a;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
 // Warp-wide sum.
 __device__ __forceinline__ float warp_sum(float x)
 {

@@ -52,28 +52,6 @@ struct RenderFwdArgs {
 constexpr int kLossCluster = 4;
 constexpr int kLossClusterTimes = 4;  // items a place of the GPU up to which clusters are used
 
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// A float of this block's shared memory layout in block `rank` of the cluster.
-__device__ __forceinline__ float ld_cluster(const float *p, int rank)
-{
-    uint32_t a;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ float sgn(float x) { return (float)((x > 0.0f) - (x < 0.0f)); }
 
 // The three float4 of list entry idx of a tile (zeros past the end).

@@ -9,7 +9,7 @@
 // Two kernels over 32 x 48 output tiles of all views.  The first stages the
 // tile plus a 5-pixel halo of both images (all three channels, coalesced) in
 // shared memory, filters the moments x, y, x^2 + y^2 and x y separably (s
-// needs the two variances only through their sum) and sums s into the loss;
+// needs the two variances only through their sum) and sums s a block;
 // per pixel and channel it writes the three partial derivatives of s with
 // respect to the moments that depend on the rendered image,
 //   ds/dmx = (2 my (a2 - a1) - 2 mx s (b2 - b1)) / (b1 b2),
@@ -17,7 +17,7 @@
 // as nine planar maps.  The second filters those maps with the same
 // (symmetric) window and adds
 //   dL/dx = g (G*ds/dmx + 2 x G*ds/dE[x^2] + y G*ds/dE[xy]),  g = -weight/(3P)
-// to d_rgb.
+// to d_rgb; a block more adds the sums of s to the loss.
 //
 // The gradient kernel stages a channel's three maps while the previous
 // channel is filtered: with the tensor memory accelerator (one 4-D box per
@@ -197,10 +197,37 @@ __device__ __forceinline__ void ssim_grad_write(const float *s_out, float *__res
     }
 }
 
+// The loss value: weight (1 - mean s).  The moment pass leaves each block's sum
+// of s in the workspace, after the maps, and one more block of the gradient pass,
+// its last, adds them up and to the loss, once: an addition a block rounds the
+// running loss each time (840 for four 641x479 views: errors up to 4.7e-6 of it,
+// by their order, against 9.7e-7).  Without room for the sums (sums null) the
+// blocks add their shares themselves.
+struct SsimLoss {
+    float *sums;  // [n], or null
+    int32_t n;    // tiles
+    float *loss;
+    double weight, inv;  // inv = 1 / (3 P)
+};
+
+__device__ __forceinline__ void ssim_add_sums(const SsimLoss &L)
+{
+    __shared__ double red[kSsimThreads / 32];
+    double acc = 0.0;
+    #pragma unroll 4
+    for (int i = threadIdx.x; i < L.n; i += kSsimThreads) acc += (double)L.sums[i];
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFullMask, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < kSsimThreads / 32; w++) acc += red[w];
+    atomicAdd(L.loss, (float)(L.weight * (1.0 - L.inv * acc)));
+}
+
 __global__ void __launch_bounds__(kSsimThreads) ssim_stats_kernel(const float *__restrict__ x,
                                                                   const float *__restrict__ y, SsimTiles T,
-                                                                  float *__restrict__ partial, float *loss,
-                                                                  float scale, float constant)
+                                                                  float *__restrict__ partial, SsimLoss L)
 {
     chain_go();
     extern __shared__ float smem[];
@@ -303,17 +330,22 @@ __global__ void __launch_bounds__(kSsimThreads) ssim_stats_kernel(const float *_
     if (tid == 0) {
         float s = 0.f;
         for (int w = 0; w < kSsimThreads / 32; w++) s += red[w];
-        atomicAdd(loss, scale * s + (blockIdx.x == 0 ? constant : 0.0f));
+        if (L.sums) L.sums[blockIdx.x] = s;
+        else atomicAdd(L.loss, (float)(-L.weight * L.inv * s + (blockIdx.x == 0 ? L.weight : 0.0)));
     }
 }
 
 __global__ void __launch_bounds__(kSsimThreads) ssim_grad_kernel(const float *__restrict__ x,
                                                                  const float *__restrict__ y, SsimTiles T,
                                                                  const float *__restrict__ partial,
-                                                                 float *__restrict__ d_rgb, float gsc)
+                                                                 float *__restrict__ d_rgb, float gsc, SsimLoss L)
 {
     chain_go();
     chain_wait();
+    if ((int)blockIdx.x == L.n) {
+        ssim_add_sums(L);
+        return;
+    }
     extern __shared__ float smem[];
     constexpr int kBuf = 3 * kSsimRows * kSsimInPitch;
     float *s_in = smem;                                 // [2][3][rows][43]: a channel's three maps, double-buffered
@@ -431,10 +463,14 @@ __global__ void __launch_bounds__(kSsimThreads, GS_SSIM_GRAD_TMA_BLOCKS) ssim_gr
                                                                      const float *__restrict__ y, SsimTiles T,
                                                                      const __grid_constant__ SsimMaps maps,
                                                                      float *__restrict__ d_rgb, float gsc,
-                                                                     uint32_t *status, uint32_t extra_tx)
+                                                                     SsimLoss L, uint32_t *status, uint32_t extra_tx)
 {
     chain_go();
     chain_wait();
+    if ((int)blockIdx.x == L.n) {
+        ssim_add_sums(L);
+        return;
+    }
     extern __shared__ __align__(128) float smem[];
     float *s_in = smem;                                 // [3][rows][52]: a channel's three maps (TMA box)
     float *s_h = smem + 3 * kSsimRows * kSsimTmaPitch;  // [3][rows][33]
@@ -653,6 +689,7 @@ using namespace gs;
 extern "C" size_t gs_ssim_workspace_size(int64_t n_pixels)
 {
     // nine maps; an eighth more for rows padded to 16 bytes (views at least 24 wide)
+    // and the blocks' sums of the loss
     return n_pixels < 0 ? 0 : sizeof(float) * 9 * ((size_t)n_pixels + (size_t)n_pixels / 8);
 }
 
@@ -673,17 +710,20 @@ static gs_status_t ssim_launch(const float *rgb, const float *target_rgb, const 
     const int blocks = T.base[n_views];
     float *partial = static_cast<float *>(workspace);
     const float scale = (float)(-(double)weight / (3.0 * (double)P));
-    // weight * (1 - mean s): block 0 adds the constant weight, every block -weight/(3P) times its sum of s
-    ssim_stats_kernel<<<blocks, kSsimThreads, kSsimStatsSmem, s>>>(rgb, target_rgb, T, partial, loss, scale, weight);
+    const bool room = workspace_bytes / sizeof(float) >= (size_t)(9 * T.n_map) + (size_t)blocks;
+    const SsimLoss L = {room ? partial + 9 * T.n_map : nullptr, blocks, loss, (double)weight, 1.0 / (3.0 * (double)P)};
+    const int grid = blocks + (room ? 1 : 0);  // the gradient pass's, with the block that adds up the loss
+    ssim_stats_kernel<<<blocks, kSsimThreads, kSsimStatsSmem, s>>>(rgb, target_rgb, T, partial, L);
     static SsimMaps maps;  // 8 KB: static, not on the stack; copied into the launch's parameters
     static std::mutex maps_mu;
     std::lock_guard<std::mutex> lock(maps_mu);
     // (the timeout check stays with the views whose rows need no padding)
     if ((extra_tx == 0 || rows_aligned(T)) && make_ssim_maps(T, partial, &maps))
-        launch_chained(ssim_grad_tma_kernel, blocks, kSsimThreads, kSsimGradTmaSmem, s, rgb, target_rgb, T, maps, d_rgb,
-                       scale, status, extra_tx);
+        launch_chained(ssim_grad_tma_kernel, grid, kSsimThreads, kSsimGradTmaSmem, s, rgb, target_rgb, T, maps, d_rgb,
+                       scale, L, status, extra_tx);
     else if (extra_tx == 0)
-        launch_chained(ssim_grad_kernel, blocks, kSsimThreads, kSsimGradSmem, s, rgb, target_rgb, T, partial, d_rgb, scale);
+        launch_chained(ssim_grad_kernel, grid, kSsimThreads, kSsimGradSmem, s, rgb, target_rgb, T, partial, d_rgb,
+                       scale, L);
     else
         return GS_ERR_UNSUPPORTED;
     return launch_status();
