@@ -25,7 +25,7 @@
 // Bound by latency and, where many views draw a Gaussian, instruction issue.
 // Warps walk only the views that draw one of their Gaussians, and only those
 // store and sum twist terms: colour 113 -> 97 us and geometry 77 -> 68 us for 1M
-// Gaussians in 8 views, 679 -> 672 and 598 -> 528 us for 4M in 16 (most Gaussians
+// Gaussians in 8 views, 679 -> 640 and 598 -> 523 us for 4M in 16 (most Gaussians
 // of a floor are drawn in few of its views).
 #include "chain.cuh"
 #include "common.cuh"
