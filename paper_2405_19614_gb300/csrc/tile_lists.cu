@@ -585,17 +585,26 @@ __global__ void __launch_bounds__(kMergeThreads) tile_merge_kernel(ListArgs a)
     }
 }
 
+// Allows the kernels `bytes` of dynamic shared memory, once a device.
+template <typename... K>
+static bool told_smem(PerDevice &allowed, size_t bytes, K... kernels)
+{
+    return allowed([&](int) {
+        const cudaFuncAttribute most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        return (... && (cudaFuncSetAttribute(kernels, most, (int)bytes) == cudaSuccess)) ? 1 : 0;
+    }) == 1;
+}
+
 template <bool PRIVATE>
 static gs_status_t launch_walks(const ListArgs &a, const ViewTable &vt, uint32_t blocks_per_view, size_t smem,
                                 cudaStream_t s)
 {
     const unsigned grid = blocks_per_view * (unsigned)vt.n_views;
-    if (smem > 48 * 1024) {
-        const cudaFuncAttribute most = cudaFuncAttributeMaxDynamicSharedMemorySize;
-        if (cudaFuncSetAttribute(tile_count_kernel<PRIVATE>, most, (int)smem) != cudaSuccess ||
-            cudaFuncSetAttribute(tile_scatter_kernel<PRIVATE>, most, (int)smem) != cudaSuccess)
-            return GS_ERR_CUDA;
-    }
+    // the limit belongs to the kernel, not to the launch: one constant, told once
+    // a device, so that no call lowers it between another thread's two launches
+    static PerDevice allowed;
+    if (smem > 48 * 1024 && !told_smem(allowed, kMaxTileSmem, tile_count_kernel<PRIVATE>, tile_scatter_kernel<PRIVATE>))
+        return GS_ERR_CUDA;
     launch_chained(tile_count_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
     launch_chained(tile_scan_kernel, 1, kScanThreads, 0, s, a, vt, !PRIVATE);
     launch_chained(tile_scatter_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
@@ -664,14 +673,8 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     if (st != GS_OK) return st;
     const uint32_t extra = (uint32_t)num_sms() * 2;
     const size_t sort_smem = sizeof(unsigned long long) * kTileChunk;
-    static PerDevice allowed;  // 1 once the device has been told of the kernel's shared memory
-    const int ok = allowed([&](int) {
-        return cudaFuncSetAttribute(tile_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem) ==
-                       cudaSuccess
-                   ? 1
-                   : 0;
-    });
-    if (!ok) return GS_ERR_CUDA;
+    static PerDevice allowed;
+    if (!told_smem(allowed, sort_smem, tile_sort_kernel)) return GS_ERR_CUDA;
     const unsigned groups = kSortBlock / kSortGroup;
     launch_chained(tile_sort_kernel, (n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s, a, n_tiles, extra);
     // (no list is longer than a view has Gaussians)
