@@ -489,9 +489,12 @@ extern "C" gs_status_t gs_bin_sort(const gs_projected_t *proj, int64_t n, const 
     // 1. drawn records sorted by depth
     const unsigned nb = (unsigned)((total + kEmitChunk - 1) / kEmitChunk);
     vis_count_kernel<<<nb, kEmitThreads, 0, s>>>(proj->tiles_touched, total, w.block_sums);
+    if ((st = launch_status()) != GS_OK) return st;
     scan_sums_kernel<<<1, 1024, 0, s>>>(w.block_sums, nb, total, n_vis, bins->status, nullptr, 1);
+    if ((st = launch_status()) != GS_OK) return st;
     vis_compact_kernel<<<nb, kEmitThreads, 0, s>>>(proj->rec, proj->tiles_touched, total, w.block_sums, w.rz[0],
                                                    w.rid[0], hist_depth);
+    if ((st = launch_status()) != GS_OK) return st;
     for (int p = 0; p < kDepthPasses; p++) {
         const int a = p & 1;
         const bool last = p + 1 == kDepthPasses;  // writes (depth bits, record id) pairs
@@ -512,13 +515,14 @@ extern "C" gs_status_t gs_bin_sort(const gs_projected_t *proj, int64_t n, const 
     const unsigned np = (unsigned)((total + kPairChunk - 1) / kPairChunk);
     const unsigned pgrid = (unsigned)(np < (unsigned)num_sms() * 8u ? np : (unsigned)num_sms() * 8u);
     pair_count_kernel<<<pgrid, kEmitThreads, 0, s>>>(w.recs, proj->tiles_touched, n_vis, w.block_sums);
+    if ((st = launch_status()) != GS_OK) return st;
     scan_sums_kernel<<<1, 1024, 0, s>>>(w.block_sums, np, cap, bins->n_pairs, bins->status, n_vis, kPairChunk);
+    if ((st = launch_status()) != GS_OK) return st;
     pair_emit_kernel<<<pgrid, kEmitThreads, 0, s>>>(w.recs, reinterpret_cast<const uint2 *>(proj->rect),
                                                   reinterpret_cast<const unsigned long long *>(proj->tile_mask),
                                                  proj->tiles_touched, n_vis, (uint32_t)n, vt, w.block_sums, cap,
                                                  buf_k[e], buf_v[e], hist_tile, tile_passes);
-    st = launch_status();
-    if (st != GS_OK) return st;
+    if ((st = launch_status()) != GS_OK) return st;
 
     // 3. stable passes over the tile id; the last writes keys and values
     if (cudaMemsetAsync(w.lb[0], 0, w.lb_bytes, s) != cudaSuccess) return GS_ERR_CUDA;

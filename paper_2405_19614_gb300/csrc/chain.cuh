@@ -22,14 +22,18 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "common.cuh"
+
 namespace gs {
 
 __device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // A launch with its attributes: chained (or not), in clusters of `cluster` blocks.
+// A call stops at the first launch that is refused: the kernels behind it read
+// what it would have written (places in a list among it).
 template <typename... P, typename... A>
-inline void launch_with(bool chained, int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+[[nodiscard]] inline gs_status_t launch_with(bool chained, int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                         cudaStream_t s, A... args)
 {
     cudaLaunchAttribute attr[2] = {};
@@ -49,13 +53,14 @@ inline void launch_with(bool chained, int cluster, void (*kernel)(P...), dim3 gr
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
-    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // errors are read by launch_status
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    return launch_status();
 }
 
 template <typename... P, typename... A>
-inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+[[nodiscard]] inline gs_status_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
 {
-    launch_with(true, 1, kernel, grid, block, smem, s, args...);
+    return launch_with(true, 1, kernel, grid, block, smem, s, args...);
 }
 
 // Clears n words for the kernel chained after it (a memset would end before that
@@ -66,10 +71,11 @@ static __global__ void chain_clear_kernel(uint32_t *p, uint32_t n)
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0u;
 }
 
-inline void launch_clear(uint32_t *p, uint32_t n, cudaStream_t s)
+[[nodiscard]] inline gs_status_t launch_clear(uint32_t *p, uint32_t n, cudaStream_t s)
 {
     const unsigned blocks = (n + 1023) / 1024;
     chain_clear_kernel<<<blocks < 512 ? blocks : 512, n < 256 ? 32 : 256, 0, s>>>(p, n);
+    return launch_status();
 }
 
 }  // namespace gs

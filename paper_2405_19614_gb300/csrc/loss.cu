@@ -78,7 +78,6 @@ extern "C" gs_status_t gs_loss_l1(const float *rgb, const float *depth, const fl
     const int sms = num_sms();
     const int64_t want = (n_pixels + kL1Threads - 1) / kL1Threads, most = (int64_t)sms * 8;
     const int64_t blocks = ((want < most ? want : most) + kL1Cluster - 1) / kL1Cluster * kL1Cluster;
-    launch_with(false, kL1Cluster, loss_l1_kernel, (unsigned)blocks, kL1Threads, 0, as_stream(stream), rgb, depth, alpha,
-                target_rgb, target_depth, n_pixels, kc, kd, use_gate, gamma, loss, d_rgb, d_depth);
-    return launch_status();
+    return launch_with(false, kL1Cluster, loss_l1_kernel, (unsigned)blocks, kL1Threads, 0, as_stream(stream), rgb, depth,
+                       alpha, target_rgb, target_depth, n_pixels, kc, kd, use_gate, gamma, loss, d_rgb, d_depth);
 }

@@ -318,8 +318,11 @@ extern "C" gs_status_t gs_densify(const float *alpha, const float *target_rgb, c
     const int64_t nb = (P + kSelChunk - 1) / kSelChunk;
     DensifySel sel{alpha, target_depth, threshold};
     select_count_kernel<<<(unsigned)nb, kSelThreads, 0, s>>>(sel, P, counts);
+    st = launch_status();
+    if (st != GS_OK) return st;
     uint32_t *total = counts + nb;
-    launch_chained(select_scan_kernel, 1, 1024, 0, s, counts, nb, total, (uint32_t)left, n_added, status);
+    st = launch_chained(select_scan_kernel, 1, 1024, 0, s, counts, nb, total, (uint32_t)left, n_added, status);
+    if (st != GS_OK) return st;
     DensifyArgs a;
     a.alpha = alpha;
     a.depth = target_depth;
@@ -336,8 +339,7 @@ extern "C" gs_status_t gs_densify(const float *alpha, const float *target_rgb, c
     a.n_old = n_old;
     a.capacity = capacity;
     a.P = P;
-    launch_chained(densify_write_kernel, dim3((unsigned)nb, kDensifySplit), kSelThreads, 0, s, a, vt, counts);
-    return launch_status();
+    return launch_chained(densify_write_kernel, dim3((unsigned)nb, kDensifySplit), kSelThreads, 0, s, a, vt, counts);
 }
 
 extern "C" gs_status_t gs_prune_select(const float *opacity_logit, int64_t n, float tau, int32_t *new_index,
@@ -355,9 +357,12 @@ extern "C" gs_status_t gs_prune_select(const float *opacity_logit, int64_t n, fl
     const int64_t nb = (n + kSelChunk - 1) / kSelChunk;
     PruneSel sel{opacity_logit, min_logit};
     select_count_kernel<<<(unsigned)nb, kSelThreads, 0, s>>>(sel, n, counts);
-    launch_chained(select_scan_kernel, 1, 1024, 0, s, counts, nb, n_kept, 0xffffffffu, nullptr, nullptr);
-    launch_chained(prune_index_kernel, (unsigned)nb, kSelThreads, 0, s, opacity_logit, n, min_logit, counts, new_index);
-    return launch_status();
+    gs_status_t st = launch_status();
+    if (st != GS_OK) return st;
+    st = launch_chained(select_scan_kernel, 1, 1024, 0, s, counts, nb, n_kept, 0xffffffffu, nullptr, nullptr);
+    if (st != GS_OK) return st;
+    return launch_chained(prune_index_kernel, (unsigned)nb, kSelThreads, 0, s, opacity_logit, n, min_logit, counts,
+                          new_index);
 }
 
 extern "C" gs_status_t gs_compact_rows(const int32_t *new_index, int64_t n, const gs_rows_t *arrays,

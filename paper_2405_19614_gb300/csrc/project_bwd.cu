@@ -705,15 +705,17 @@ static gs_status_t project_bwd(const gs_params_t *params, const gs_view_t *views
     cudaStream_t s = as_stream(stream);
     // colour first: the geometry kernel clears the 2D gradients after use
     const unsigned cblocks = (unsigned)((params->n + kColorThreads - 1) / kColorThreads);
+    auto colour = project_bwd_color_kernel<3>;
     switch (params->sh_degree) {
-    case 0: launch_with(chained, 1, project_bwd_color_kernel<0>, cblocks, kColorThreads, 0, s, a, vt); break;
-    case 1: launch_with(chained, 1, project_bwd_color_kernel<1>, cblocks, kColorThreads, 0, s, a, vt); break;
-    case 2: launch_with(chained, 1, project_bwd_color_kernel<2>, cblocks, kColorThreads, 0, s, a, vt); break;
-    default: launch_with(chained, 1, project_bwd_color_kernel<3>, cblocks, kColorThreads, 0, s, a, vt); break;
+    case 0: colour = project_bwd_color_kernel<0>; break;
+    case 1: colour = project_bwd_color_kernel<1>; break;
+    case 2: colour = project_bwd_color_kernel<2>; break;
+    default: break;
     }
+    st = launch_with(chained, 1, colour, cblocks, kColorThreads, 0, s, a, vt);
+    if (st != GS_OK) return st;
     const unsigned gblocks = (unsigned)((params->n + threads - 1) / threads);
-    launch_chained(project_bwd_geom_kernel, gblocks, threads, 0, s, a, vt);
-    return launch_status();
+    return launch_chained(project_bwd_geom_kernel, gblocks, threads, 0, s, a, vt);
 }
 
 extern "C" gs_status_t gs_project_bwd(const gs_params_t *params, const gs_view_t *views, const float *viewmats,

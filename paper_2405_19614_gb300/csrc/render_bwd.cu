@@ -575,10 +575,13 @@ static gs_status_t launch_bwd(RenderBwdArgs a, ViewTable vt, const CUtensorMap &
     // every item has a warp of its own when the grid holds them all: no counter
     // to clear and none to wait for (2 us less of a small image)
     const bool counted = blocks_needed > slots;
-    if (counted) launch_clear(a.work_counter, 1, s);
-    else a.work_counter = nullptr;
-    launch_with(counted, 1, kern, grid > 0 ? grid : 1, kRenderThreads, 0, s, a, vt, map);
-    return launch_status();
+    if (counted) {
+        const gs_status_t st = launch_clear(a.work_counter, 1, s);
+        if (st != GS_OK) return st;
+    } else {
+        a.work_counter = nullptr;
+    }
+    return launch_with(counted, 1, kern, grid > 0 ? grid : 1, kRenderThreads, 0, s, a, vt, map);
 }
 
 template <int CH, bool TMA, bool ASYNC = false>

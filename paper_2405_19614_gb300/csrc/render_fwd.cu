@@ -463,12 +463,15 @@ static gs_status_t launch_fwd(RenderFwdArgs a, ViewTable vt, const CUtensorMap &
     // every item has a warp of its own when the grid holds them all: no counter
     // to clear and none to wait for (2 us less of a small image)
     const bool counted = blocks_needed > slots;
-    if (counted) launch_clear(a.work_counter, 1, s);
-    else a.work_counter = nullptr;
+    if (counted) {
+        const gs_status_t st = launch_clear(a.work_counter, 1, s);
+        if (st != GS_OK) return st;
+    } else {
+        a.work_counter = nullptr;
+    }
     a.loss_cluster = LOSS && blocks_needed < kLossClusterTimes * slots ? kLossCluster : 1;
     const int blocks = (grid > 0 ? grid + a.loss_cluster - 1 : a.loss_cluster) / a.loss_cluster * a.loss_cluster;
-    launch_with(counted, a.loss_cluster, kern, blocks, kRenderThreads, 0, s, a, vt, map);
-    return launch_status();
+    return launch_with(counted, a.loss_cluster, kern, blocks, kRenderThreads, 0, s, a, vt, map);
 }
 
 template <int CH, bool TMA, bool STATS, bool LOSS, bool ASYNC = false>

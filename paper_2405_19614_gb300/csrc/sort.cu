@@ -328,6 +328,8 @@ extern "C" gs_status_t gs_check_lookback_timeout(uint32_t spin_limit, int32_t wi
     if (cudaMemsetAsync(ws + CheckLayout::hist, 0, CheckLayout::bytes - CheckLayout::hist, s) != cudaSuccess)
         return GS_ERR_CUDA;
     check_fill_kernel<<<kCheckKeys / 256, 256, 0, s>>>(ws, withhold_first_tile != 0);
+    const gs_status_t st = launch_status();
+    if (st != GS_OK) return st;
     const SortExpand none = {};
     auto u32 = [&](size_t off) { return reinterpret_cast<uint32_t *>(ws + off); };
     launch_pass<kSortPlain>(u32(CheckLayout::kin), u32(CheckLayout::vin), u32(CheckLayout::kout),

@@ -189,12 +189,15 @@ extern "C" gs_status_t gs_spatial_order(const float *means, int64_t n, int32_t *
     const unsigned blocks = (unsigned)((n + kSpThreads - 1) / kSpThreads);
     const unsigned bb = blocks < (unsigned)num_sms() * 4 ? blocks : (unsigned)num_sms() * 4;
     bbox_kernel<<<bb, kSpThreads, 0, s>>>(means, n, box);
+    gs_status_t st = launch_status();
+    if (st != GS_OK) return st;
     morton_kernel<<<bb, kSpThreads, 0, s>>>(means, n, box, w.keys[0], w.idx[0], hist, n_dev);
+    if ((st = launch_status()) != GS_OK) return st;
     for (int p = 0; p < kSpPasses; p++) {
         const int a = p & 1;
-        gs_status_t st = onesweep_pass(w.keys[a], w.idx[a], w.keys[a ^ 1], w.idx[a ^ 1], n_dev, n, hist + p * kRadix,
-                                       w.lb[a], p + 1 < kSpPasses ? w.lb[a ^ 1] : nullptr, counters + p, 8 * p,
-                                       kSortPlain, nullptr, status, s);
+        st = onesweep_pass(w.keys[a], w.idx[a], w.keys[a ^ 1], w.idx[a ^ 1], n_dev, n, hist + p * kRadix, w.lb[a],
+                           p + 1 < kSpPasses ? w.lb[a ^ 1] : nullptr, counters + p, 8 * p, kSortPlain, nullptr, status,
+                           s);
         if (st != GS_OK) return st;
     }
     rank_kernel<<<blocks, kSpThreads, 0, s>>>(w.idx[0], n, new_index);  // an even number of passes ends in 0

@@ -714,19 +714,19 @@ static gs_status_t ssim_launch(const float *rgb, const float *target_rgb, const 
     const SsimLoss L = {room ? partial + 9 * T.n_map : nullptr, blocks, loss, (double)weight, 1.0 / (3.0 * (double)P)};
     const int grid = blocks + (room ? 1 : 0);  // the gradient pass's, with the block that adds up the loss
     ssim_stats_kernel<<<blocks, kSsimThreads, kSsimStatsSmem, s>>>(rgb, target_rgb, T, partial, L);
+    st = launch_status();
+    if (st != GS_OK) return st;
     static SsimMaps maps;  // 8 KB: static, not on the stack; copied into the launch's parameters
     static std::mutex maps_mu;
     std::lock_guard<std::mutex> lock(maps_mu);
     // (the timeout check stays with the views whose rows need no padding)
     if ((extra_tx == 0 || rows_aligned(T)) && make_ssim_maps(T, partial, &maps))
-        launch_chained(ssim_grad_tma_kernel, grid, kSsimThreads, kSsimGradTmaSmem, s, rgb, target_rgb, T, maps, d_rgb,
-                       scale, L, status, extra_tx);
-    else if (extra_tx == 0)
-        launch_chained(ssim_grad_kernel, grid, kSsimThreads, kSsimGradSmem, s, rgb, target_rgb, T, partial, d_rgb,
-                       scale, L);
-    else
-        return GS_ERR_UNSUPPORTED;
-    return launch_status();
+        return launch_chained(ssim_grad_tma_kernel, grid, kSsimThreads, kSsimGradTmaSmem, s, rgb, target_rgb, T, maps,
+                              d_rgb, scale, L, status, extra_tx);
+    if (extra_tx == 0)
+        return launch_chained(ssim_grad_kernel, grid, kSsimThreads, kSsimGradSmem, s, rgb, target_rgb, T, partial, d_rgb,
+                              scale, L);
+    return GS_ERR_UNSUPPORTED;
 }
 
 extern "C" gs_status_t gs_loss_ssim(const float *rgb, const float *target_rgb, const gs_view_t *views,

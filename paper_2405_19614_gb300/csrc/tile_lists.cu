@@ -605,10 +605,11 @@ static gs_status_t launch_walks(const ListArgs &a, const ViewTable &vt, uint32_t
     static PerDevice allowed;
     if (smem > 48 * 1024 && !told_smem(allowed, kMaxTileSmem, tile_count_kernel<PRIVATE>, tile_scatter_kernel<PRIVATE>))
         return GS_ERR_CUDA;
-    launch_chained(tile_count_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
-    launch_chained(tile_scan_kernel, 1, kScanThreads, 0, s, a, vt, !PRIVATE);
-    launch_chained(tile_scatter_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
-    return launch_status();
+    gs_status_t st = launch_chained(tile_count_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
+    if (st != GS_OK) return st;
+    st = launch_chained(tile_scan_kernel, 1, kScanThreads, 0, s, a, vt, !PRIVATE);
+    if (st != GS_OK) return st;
+    return launch_chained(tile_scatter_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
 }
 
 // Where a tile's list could grow very long, its chunks' merge (a search in
@@ -644,7 +645,8 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     a.keys = bins->keys;
     a.vals = bins->vals;
     const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
-    launch_clear(reinterpret_cast<uint32_t *>(a.ranges), 2 * n_tiles, s);
+    gs_status_t st = launch_clear(reinterpret_cast<uint32_t *>(a.ranges), 2 * n_tiles, s);
+    if (st != GS_OK) return st;
     uint32_t most_tiles = 0;
     for (int v = 0; v < vt.n_views; v++) {
         const uint32_t t = (uint32_t)(vt.v[v].tiles_x * vt.v[v].tiles_y);
@@ -659,7 +661,6 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     const size_t smem = sizeof(uint32_t) * most_tiles;
     const int64_t rows = (int64_t)(buf.table_bytes / smem) / vt.n_views;  // table rows a view
     const bool priv = smem <= kMaxTileSmem && (rows >= per_view || rows * vt.n_views >= num_sms());
-    gs_status_t st;
     if (priv) {
         per_view = per_view < rows ? per_view : rows;
         a.table = static_cast<uint32_t *>(buf.table);
@@ -676,10 +677,11 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     static PerDevice allowed;
     if (!told_smem(allowed, sort_smem, tile_sort_kernel)) return GS_ERR_CUDA;
     const unsigned groups = kSortBlock / kSortGroup;
-    launch_chained(tile_sort_kernel, (n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s, a, n_tiles, extra);
+    st = launch_chained(tile_sort_kernel, (n_tiles + groups - 1) / groups + extra, kSortBlock, sort_smem, s, a, n_tiles,
+                        extra);
     // (no list is longer than a view has Gaussians)
-    if (n > kTileChunk) launch_chained(tile_merge_kernel, (unsigned)num_sms() * 8, kMergeThreads, 0, s, a);
-    return launch_status();
+    if (st != GS_OK || n <= kTileChunk) return st;
+    return launch_chained(tile_merge_kernel, (unsigned)num_sms() * 8, kMergeThreads, 0, s, a);
 }
 
 }  // namespace gs
