@@ -1,4 +1,4 @@
-// a2 - a4 for maps that are not crowded into a few tiles: the tile lists by
+// a2 - a4 for maps of up to 2,048 records a tile on average: the tile lists by
 // counting, scattering and sorting each tile on its own.
 //
 //   1. tile_count_kernel adds up each tile's pairs and tile_scan_kernel turns
@@ -11,8 +11,8 @@
 //      depend on the order they arrived in: it is the list a stable sort of
 //      the 64-bit keys (tile << 32) | depth bits gives;
 //   4. tile_merge_kernel puts together the chunks of the tiles of more than
-//      kTileChunk words (a rank by binary search in the other chunks); it has
-//      nothing to do on most calls.
+//      kTileChunk words, spread over the GPU however few such tiles there are;
+//      it has nothing to do on most calls.
 //
 // Against sorting all records by depth, emitting their pairs in that order and
 // sorting the pairs by tile id (binning.cu: 13 to 16 dependent launches, of
@@ -24,7 +24,12 @@
 //   100k Gaussians, 640x480, 49k pairs            36 against 125 us
 //   300k Gaussians, 1200x680, 174k pairs          42 against 111 us
 //   1M, 8 views of 1200x680 (32x16 tiles), 4.0M   235 against 305 us
-//   4M, 16 views (lists up to 59,000), 28.2M      1.67 against 2.36 ms
+//   4M, 16 views (lists up to 59,000), 28.2M      1.51 against 2.36 ms
+// and whole calls on a map crowded into a few tiles:
+//   100k in one tile of 640x480                   150 against 144 us
+//   300k in 16 tiles of 1200x680                  124 against 152 us
+//   1M in one tile of 1200x680, in four           215, 207 against 217, 220 us
+//   4M in four tiles of 1200x680, in one          527, 848 against 558, 560 us
 #include "binning.cuh"
 #include "chain.cuh"
 #include "common.cuh"
@@ -35,11 +40,24 @@ constexpr int kListThreads = 256;
 constexpr int kSortGroup = 128;                    // threads that sort a tile
 constexpr int kSortBlock = 4 * kSortGroup;         // threads of a block: four tiles, or a long tile's chunk
 constexpr int kMergeThreads = 256;
+constexpr int kMergePer = 8;                       // words a thread of the merge sorts
+constexpr uint32_t kMergeWords = kMergeThreads * kMergePer;
+constexpr uint32_t kMergeParts = 5;                // blocks that share a chunk's part of the sorted tile
+constexpr uint32_t kMergeSlack = 128;              // how far a cut may lie from its rank
+// Chunks of a tile up to which the merge searches for each word's rank in the
+// other chunks (beyond, it sorts parts of the tile again).  8M words in lists of
+// two to six chunks took 583, 630, 700, 749 and 804 us of binning by search against
+// 872 to 885; 100k in two lists of seven 142 against 150.
+constexpr uint32_t kSearchChunks = 6;
+constexpr int kSearchAhead = 4;                    // searches a thread makes side by side
+constexpr int kCutThreads = kMergeThreads / 2;     // threads that look for a cut
+constexpr int kCutKept = 4;                        // chunks a thread follows
 constexpr int kScanThreads = 1024;
 constexpr int kBlocksPerSm = 6;                    // counting and scattering blocks, resident
 constexpr size_t kMaxTileSmem = 64 * 1024;         // a view's tiles in shared memory (16,384)
 constexpr uint32_t kGroupWords = 16 * kSortGroup;  // words a group sorts (16 KB of shared memory)
 constexpr uint32_t kTileChunk = 16 * kSortBlock;   // words a block sorts (64 KB)
+static_assert(kTileChunk / kMergeParts + 1 + 2 * kMergeSlack <= kMergeWords, "a part of a chunk and both slacks fit");
 
 // Words of the small region this path uses.
 struct ListState {
@@ -91,23 +109,51 @@ __device__ __forceinline__ bool pair_kept(const ListState &st, const Splat &s, u
     return pair_ordinal(s, i) < st.cut_pairs;
 }
 
-// What a walk does with tile i of splat s, tile `tile` of the view.
+// What a walk does with tile i of splat s, tile `tile` of the view; alone: the
+// lanes of a warp are at tiles of different splats, which may be the same.
 struct CountPut {
-    uint32_t *count;  // the view's tiles, stride words apart
-    uint32_t stride;
-    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &, uint32_t) const
+    uint32_t *count;  // the view's tiles
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &, uint32_t, bool) const
     {
-        atomicAdd(count + tile * stride, 1u);
+        atomicAdd(count + tile, 1u);
     }
 };
 
 struct ScatterPut {
     uint32_t *slot;
-    uint32_t stride;
     unsigned long long *words;
-    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t) const
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t, bool) const
     {
-        words[atomicAdd(slot + tile * stride, 1u)] = ((unsigned long long)s.z << 32) | s.idx;
+        words[atomicAdd(slot + tile, 1u)] = ((unsigned long long)s.z << 32) | s.idx;
+    }
+};
+
+// The same in the ranges' ends, where the additions of a crowded tile wait for
+// one another: lanes alone at the same tile add together.
+__device__ __forceinline__ uint32_t add_to_end(uint2 *ranges, uint32_t tile, bool alone)
+{
+    if (!alone) return atomicAdd(&ranges[tile].y, 1u);
+    const uint32_t same = __match_any_sync(__activemask(), tile);
+    const int lane = threadIdx.x & 31, leader = __ffs(same) - 1;
+    uint32_t at = 0;
+    if (lane == leader) at = atomicAdd(&ranges[tile].y, (uint32_t)__popc(same));
+    return __shfl_sync(same, at, leader) + __popc(same & ((1u << lane) - 1u));
+}
+
+struct GlobalCountPut {
+    uint2 *ranges;
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &, uint32_t, bool alone) const
+    {
+        add_to_end(ranges, tile, alone);
+    }
+};
+
+struct GlobalScatterPut {
+    uint2 *ranges;
+    unsigned long long *words;
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t, bool alone) const
+    {
+        words[add_to_end(ranges, tile, alone)] = ((unsigned long long)s.z << 32) | s.idx;
     }
 };
 
@@ -117,7 +163,7 @@ struct CutPut {
     ListState cut;
     uint2 *ranges;
     unsigned long long *words;
-    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t i) const
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t i, bool) const
     {
         if (!pair_kept(cut, s, i)) return;
         const uint32_t pos = atomicAdd(&ranges[tile].y, 1u);
@@ -171,7 +217,7 @@ __device__ __forceinline__ void walk_view(const ListArgs &a, const ViewInfo &V, 
                     const uint32_t i = (uint32_t)__ffsll((long long)m) - 1u;
                     m &= m - 1ull;
                     const uint32_t ky = (i * recip) >> 16;
-                    put(s.tile0 + ky * tiles_x + (i - ky * w), s, i);
+                    put(s.tile0 + ky * tiles_x + (i - ky * w), s, i, true);
                 }
             }
             // two of the larger records at a time, half a warp each
@@ -194,7 +240,7 @@ __device__ __forceinline__ void walk_view(const ListArgs &a, const ViewInfo &V, 
                 const uint32_t qw = q.wh & 0xffffu, tiles = have ? qw * (q.wh >> 16) : 0u;
                 for (uint32_t i = lane & 15; i < tiles; i += 16) {
                     const uint32_t ky = tiles <= 64 ? (i * inv) >> 16 : i / qw;
-                    if (tiles > 64 || ((q.mask >> i) & 1ull)) put(q.tile0 + ky * tiles_x + (i - ky * qw), q, i);
+                    if (tiles > 64 || ((q.mask >> i) & 1ull)) put(q.tile0 + ky * tiles_x + (i - ky * qw), q, i, false);
                 }
                 __syncwarp();
             }
@@ -354,9 +400,11 @@ __global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_count_kernel(
         __syncthreads();
     }
     chain_wait();
-    walk_view<false>(a, V, v, b * (kListThreads / 32) + threadIdx.x / 32, blocks_per_view * (kListThreads / 32),
-                     PRIVATE ? CountPut{s_tile, 1u} : CountPut{&ranges[0].y, 2u});
-    if (PRIVATE) {
+    const uint32_t first = b * (kListThreads / 32) + threadIdx.x / 32, stride = blocks_per_view * (kListThreads / 32);
+    if (!PRIVATE) {
+        walk_view<false>(a, V, v, first, stride, GlobalCountPut{ranges});
+    } else {
+        walk_view<false>(a, V, v, first, stride, CountPut{s_tile});
         __syncthreads();
         uint32_t *row = a.table + (size_t)blockIdx.x * a.table_pitch;
         // four additions in flight a thread; the blocks start at different
@@ -405,9 +453,9 @@ __global__ void __launch_bounds__(kListThreads, kBlocksPerSm) tile_scatter_kerne
         #pragma unroll 4
         for (uint32_t t = threadIdx.x; t < tiles; t += kListThreads) s_tile[t] = ranges[t].x + row[t];
         __syncthreads();
-        walk_view<true>(a, V, v, first, stride, ScatterPut{s_tile, 1u, a.words});
+        walk_view<true>(a, V, v, first, stride, ScatterPut{s_tile, a.words});
     } else if (!st.cut) {
-        walk_view<true>(a, V, v, first, stride, ScatterPut{&ranges[0].y, 2u, a.words});
+        walk_view<true>(a, V, v, first, stride, GlobalScatterPut{ranges, a.words});
     } else {
         walk_view<true>(a, V, v, first, stride, CutPut{st, ranges, a.words});
     }
@@ -550,38 +598,217 @@ __global__ void __launch_bounds__(kSortBlock, 2) tile_sort_kernel(ListArgs a, ui
     }
 }
 
-// Each word of a listed chunk goes to its rank in the tile: its place in its
-// own chunk plus the words below it in the tile's other chunks.
-__global__ void __launch_bounds__(kMergeThreads) tile_merge_kernel(ListArgs a)
+// Words of the sorted run below x; lo and hi bound the answer.
+__device__ __forceinline__ uint32_t words_below(const unsigned long long *run, uint32_t lo, uint32_t hi,
+                                                unsigned long long x)
+{
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (run[mid] < x) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// A value with rank words of the tile below it, give or take kMergeSlack: by a
+// search over values, interpolated and halved in turn, with kCutThreads threads
+// that follow the answer in the tile's sorted chunks (kCutKept each; the chunks
+// beyond, of a list of over 4.2M words, start afresh every time: 6M words in one
+// tile 1.80 ms against 0.76 by the radix path).  A thread's searches side by side
+// instead of one after another: 896 against 848 us for 4M words in one tile.  The words are distinct, so halving alone
+// ends with the exact rank in 64 steps; with depths spread over the list it takes
+// four to eight.  It is a function of the chunks and the rank only: the blocks on both
+// sides of a cut find the same one.  bar: a barrier of the threads' own.
+__device__ __noinline__ unsigned long long cut_value(const unsigned long long *w, uint32_t m, uint32_t chunks,
+                                                     uint32_t rank, int tid, int bar, unsigned long long (*red)[4])
+{
+    if (rank == 0) return 0ull;
+    if (rank >= m) return ~0ull;
+    auto sync = [bar]() { asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(kCutThreads) : "memory"); };
+    const int lane = tid & 31, warp = tid >> 5;
+    uint32_t lo[kCutKept], hi[kCutKept];
+    unsigned long long a = ~0ull, b = 0ull;  // the smallest word, and one above the largest
+    #pragma unroll
+    for (int k = 0; k < kCutKept; k++) {
+        const uint32_t c = tid + k * kCutThreads;
+        lo[k] = 0;
+        hi[k] = c < chunks ? min(kTileChunk, m - c * kTileChunk) : 0u;
+    }
+    for (uint32_t c = tid; c < chunks; c += kCutThreads) {
+        a = min(a, w[c * kTileChunk]);
+        b = max(b, w[min(m, (c + 1) * kTileChunk) - 1] + 1);
+    }
+    #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a = min(a, __shfl_xor_sync(kFullMask, a, o));
+        b = max(b, __shfl_xor_sync(kFullMask, b, o));
+    }
+    if (lane == 0) {
+        red[0][warp] = a;
+        red[1][warp] = b;
+    }
+    sync();
+    a = min(min(red[0][0], red[0][1]), min(red[0][2], red[0][3]));
+    b = max(max(red[1][0], red[1][1]), max(red[1][2], red[1][3]));
+    uint32_t ra = 0, rb = m;  // words below a (at most rank) and below b (more than rank)
+    #pragma unroll 1
+    for (int step = 0; step < 132 && b - a > 1; step++) {
+        unsigned long long x = a + ((b - a) >> 1);
+        if (!(step & 1)) {
+            x = a + (unsigned long long)((float)(b - a) * ((float)(rank - ra) / (float)(rb - ra)));
+            x = min(max(x, a + 1), b - 1);
+        }
+        uint32_t at[kCutKept], r = 0;
+        #pragma unroll
+        for (int k = 0; k < kCutKept; k++) {
+            at[k] = words_below(w + (size_t)(tid + k * kCutThreads) * kTileChunk, lo[k], hi[k], x);
+            r += at[k];
+        }
+        for (uint32_t c = tid + kCutKept * kCutThreads; c < chunks; c += kCutThreads)
+            r += words_below(w + (size_t)c * kTileChunk, 0u, min(kTileChunk, m - c * kTileChunk), x);
+        r = __reduce_add_sync(kFullMask, r);
+        unsigned long long *part = red[2 + (step & 1)];  // (written again two barriers later)
+        if (lane == 0) part[warp] = r;
+        sync();
+        r = (uint32_t)(part[0] + part[1] + part[2] + part[3]);
+        if (r <= rank) {
+            if (rank - r <= kMergeSlack) return x;
+            a = x;
+            ra = r;
+        } else {
+            if (r - rank <= kMergeSlack) return x;
+            b = x;
+            rb = r;
+        }
+        #pragma unroll
+        for (int k = 0; k < kCutKept; k++) {
+            if (r <= rank) lo[k] = at[k];
+            else hi[k] = at[k];
+        }
+    }
+    return a;
+}
+
+// Words [first, end) of a tile's chunk tc.y to their ranks in the tile: the place
+// in the chunk plus the words below in the other chunks, kSearchAhead words at a time.
+__device__ __forceinline__ void rank_words(const ListArgs &a, uint2 tc, uint2 r, uint32_t m, uint32_t chunks,
+                                           uint32_t first, uint32_t end, int tid)
+{
+    const unsigned long long *w = a.words + r.x;
+    for (uint32_t i0 = first + tid; i0 < end; i0 += kSearchAhead * kMergeThreads) {
+        unsigned long long x[kSearchAhead];
+        uint32_t rank[kSearchAhead];
+        #pragma unroll
+        for (int u = 0; u < kSearchAhead; u++) {
+            const uint32_t i = i0 + u * kMergeThreads;
+            x[u] = i < end ? w[i] : 0ull;
+            rank[u] = i - tc.y * kTileChunk;
+        }
+        for (uint32_t c = 0; c < chunks; c++) {
+            if (c == tc.y) continue;
+            const unsigned long long *run = w + c * kTileChunk;
+            uint32_t lo[kSearchAhead] = {};
+            uint32_t n = min(kTileChunk, m - c * kTileChunk);
+            while (n > 1) {
+                const uint32_t half = n >> 1;
+                #pragma unroll
+                for (int u = 0; u < kSearchAhead; u++) lo[u] += run[lo[u] + half - 1] < x[u] ? half : 0u;
+                n -= half;
+            }
+            #pragma unroll
+            for (int u = 0; u < kSearchAhead; u++) rank[u] += lo[u] + (run[lo[u]] < x[u] ? 1u : 0u);
+        }
+        #pragma unroll
+        for (int u = 0; u < kSearchAhead; u++) {
+            if (i0 + u * kMergeThreads >= end) continue;
+            a.keys[r.x + rank[u]] = ((uint64_t)tc.x << 32) | (x[u] >> 32);
+            a.vals[r.x + rank[u]] = (uint32_t)x[u];
+        }
+    }
+}
+
+// The tiles of several sorted chunks.  A block takes a fifth of a chunk: of up to
+// kSearchChunks chunks, the words at those places, each to its rank; of more, the
+// words of those ranks: it finds the values that cut the tile in front of and
+// behind them, gathers what lies in between from all chunks and sorts it again, so
+// that a word's work does not grow with the list but for the cuts (a few searches
+// in every chunk for 1,638 words).  Bound by the latency of the searches' loads.
+// One list of 1M words: 80 us (8.3 ms when a block searched for a whole chunk's
+// words, one by one, in all other chunks), of 100k 55 (450); the 28.2M pairs of a
+// 4M-Gaussian floor 154 (334).
+__global__ void __launch_bounds__(kMergeThreads, 4) tile_merge_kernel(ListArgs a)
 {
     chain_go();
     chain_wait();
-    const uint32_t n_long = a.state->n_long;
-    for (uint32_t j = blockIdx.x; j < n_long; j += gridDim.x) {
-        const uint2 tc = a.long_chunks[j];
+    __shared__ unsigned long long s[kMergeWords];
+    __shared__ unsigned long long s_red[2][4][4], s_cut[2];
+    __shared__ uint32_t s_end[kMergeThreads], s_src[kMergeThreads], s_sum[2][kMergeThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t items = a.state->n_long * kMergeParts;
+    for (uint32_t q = blockIdx.x; q < items; q += gridDim.x) {
+        const uint2 tc = a.long_chunks[q / kMergeParts];
         const uint2 r = a.ranges[tc.x];
-        const uint32_t m = r.y - r.x, chunks = (m + kTileChunk - 1) / kTileChunk;
-        if (chunks == 1) continue;  // finished by the sort
+        const uint32_t m = r.y - r.x, chunks = (m + kTileChunk - 1) / kTileChunk, part = q % kMergeParts;
+        const uint32_t first = tc.y * kTileChunk + part * kTileChunk / kMergeParts;
+        if (chunks == 1 || first >= m) continue;  // finished by the sort, or behind the last word
+        const uint32_t end = tc.y * kTileChunk + (part + 1) * kTileChunk / kMergeParts;
         const unsigned long long *w = a.words + r.x;
-        const uint32_t lo0 = tc.y * kTileChunk, hi0 = min(m, lo0 + kTileChunk);
-        for (uint32_t i = lo0 + threadIdx.x; i < hi0; i += kMergeThreads) {
-            const unsigned long long x = w[i];
-            uint32_t rank = i - lo0;
-            for (uint32_t c = 0; c < chunks; c++) {
-                if (c == tc.y) continue;
-                const unsigned long long *run = w + c * kTileChunk;
-                uint32_t lo = 0, n = min(kTileChunk, m - c * kTileChunk);
-                while (n > 0) {
-                    const uint32_t half = n >> 1;
-                    const bool below = run[lo + half] < x;
-                    lo = below ? lo + half + 1 : lo;
-                    n = below ? n - half - 1 : half;
-                }
-                rank += lo;
-            }
-            a.keys[r.x + rank] = ((uint64_t)tc.x << 32) | (x >> 32);
-            a.vals[r.x + rank] = (uint32_t)x;
+        if (chunks <= kSearchChunks) {
+            rank_words(a, tc, r, m, chunks, first, min(end, m), tid);
+            continue;
         }
+        {
+            const int g = tid / kCutThreads;
+            const unsigned long long x = cut_value(w, m, chunks, g ? end : first, tid % kCutThreads, 1 + g, s_red[g]);
+            if (tid % kCutThreads == 0) s_cut[g] = x;
+        }
+        __syncthreads();
+        const unsigned long long from = s_cut[0], to = s_cut[1];
+        uint32_t have = 0, before = 0;  // words gathered; words below `from` in this thread's chunks
+        for (uint32_t c0 = 0; c0 < chunks; c0 += kMergeThreads) {
+            const uint32_t c = c0 + tid;
+            uint32_t lo = 0, n = 0;
+            if (c < chunks) {
+                const unsigned long long *run = w + (size_t)c * kTileChunk;
+                const uint32_t len = min(kTileChunk, m - c * kTileChunk);
+                lo = words_below(run, 0u, len, from);
+                n = words_below(run, lo, len, to) - lo;
+            }
+            before += lo;
+            uint32_t inc = n;
+            #pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFullMask, inc, o);
+                if (lane >= o) inc += y;
+            }
+            if (lane == 31) s_sum[0][warp] = inc;
+            __syncthreads();
+            for (int k = 0; k < warp; k++) inc += s_sum[0][k];
+            s_end[tid] = inc;
+            s_src[tid] = c * kTileChunk + lo - (inc - n);  // word i of the gathered ones: w[s_src + i]
+            __syncthreads();
+            const uint32_t here = s_end[kMergeThreads - 1];
+            for (uint32_t i = tid; i < here; i += kMergeThreads) {
+                uint32_t k = 0;  // the first chunk that ends behind word i
+                #pragma unroll
+                for (uint32_t half = kMergeThreads / 2; half > 0; half >>= 1) k += s_end[k + half - 1] <= i ? half : 0u;
+                if (have + i < kMergeWords) s[have + i] = w[s_src[k] + i];  // (always: see kMergeWords)
+            }
+            have += here;
+            __syncthreads();
+        }
+        have = min(have, kMergeWords);
+        before = __reduce_add_sync(kFullMask, before);
+        if (lane == 0) s_sum[1][warp] = before;
+        group_sort<kMergePer, kMergeThreads>(s, have, s, tid, []() { __syncthreads(); });
+        uint32_t out = r.x;
+        for (int k = 0; k < kMergeThreads / 32; k++) out += s_sum[1][k];
+        for (uint32_t i = tid; i < have; i += kMergeThreads) {
+            const unsigned long long x = s[i];
+            a.keys[out + i] = ((uint64_t)tc.x << 32) | (x >> 32);
+            a.vals[out + i] = (uint32_t)x;
+        }
+        __syncthreads();
     }
 }
 
@@ -681,7 +908,7 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
                         extra);
     // (no list is longer than a view has Gaussians)
     if (st != GS_OK || n <= kTileChunk) return st;
-    return launch_chained(tile_merge_kernel, (unsigned)num_sms() * 8, kMergeThreads, 0, s, a);
+    return launch_chained(tile_merge_kernel, (unsigned)num_sms() * 4, kMergeThreads, 0, s, a);
 }
 
 }  // namespace gs
