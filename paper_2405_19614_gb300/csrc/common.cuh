@@ -161,13 +161,22 @@ __device__ __forceinline__ uint32_t cluster_rank()
     return r;
 }
 
-// A float of this block's shared memory layout in block `rank` of the cluster.
+// A value of this block's shared memory layout in block `rank` of the cluster.
 __device__ __forceinline__ float ld_cluster(const float *p, int rank)
 {
     uint32_t a;
     float v;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ unsigned long long ld_cluster(const unsigned long long *p, int rank)
+{
+    uint32_t a;
+    unsigned long long v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
     return v;
 }
 

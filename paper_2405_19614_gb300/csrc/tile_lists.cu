@@ -53,6 +53,14 @@ constexpr int kSearchAhead = 4;                    // searches a thread makes si
 constexpr int kCutThreads = kMergeThreads / 2;     // threads that look for a cut
 constexpr int kCutKept = 4;                        // chunks a thread follows
 constexpr int kScanThreads = 1024;
+// Records up to which the pairs beyond the capacity are cut in the scan kernel, by
+// a cluster of kCutCluster blocks: a call that cuts nothing pays 0.3 to 1.5 us for
+// the cluster's launch (300k-Gaussian render, 100k-Gaussian tracking step; as much with
+// four blocks).  A launch a step, over the whole GPU, cuts faster but costs every
+// call 4 to 7 us: 300k records, 333k pairs at a capacity of 3/4, 192 against 106 us,
+// 1M 403 against 155.
+constexpr int kCutCluster = 8;
+constexpr uint32_t kCutInScan = 1u << 20;
 constexpr int kBlocksPerSm = 6;                    // counting and scattering blocks, resident
 constexpr size_t kMaxTileSmem = 64 * 1024;         // a view's tiles in shared memory (16,384)
 constexpr uint32_t kGroupWords = 16 * kSortGroup;  // words a group sorts (16 KB of shared memory)
@@ -61,10 +69,12 @@ static_assert(kTileChunk / kMergeParts + 1 + 2 * kMergeSlack <= kMergeWords, "a 
 
 // Words of the small region this path uses.
 struct ListState {
+    uint64_t room;       // pairs that still fit, while the cut is looked for
     uint32_t n_long;     // chunks listed in long_chunks
     uint32_t cut;        // 1: the pairs exceed the capacity and only the nearest are kept
     uint32_t cut_z, cut_r;  // (depth bits, record id) of the last record kept
     uint32_t cut_pairs;  // how many of its pairs
+    uint32_t arrived;    // blocks that are done with a step of the cut
 };
 
 struct ListArgs {
@@ -80,6 +90,7 @@ struct ListArgs {
     uint2 *long_chunks;         // (tile, chunk of kTileChunk) of the tiles longer than kGroupWords
     unsigned long long *words;  // [cap] unsorted (depth bits, index)
     uint32_t *table;  // [blocks][table_pitch] a block's first slot in each tile of its view
+    unsigned long long *cut_hist;  // [kCutBins] of a cut by several launches (then there is no table)
     uint32_t table_pitch;
     uint64_t *keys;
     uint32_t *vals;
@@ -163,10 +174,10 @@ struct CutPut {
     ListState cut;
     uint2 *ranges;
     unsigned long long *words;
-    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t i, bool) const
+    __device__ __forceinline__ void operator()(uint32_t tile, const Splat &s, uint32_t i, bool alone) const
     {
         if (!pair_kept(cut, s, i)) return;
-        const uint32_t pos = atomicAdd(&ranges[tile].y, 1u);
+        const uint32_t pos = add_to_end(ranges, tile, alone);
         if (words) words[pos] = ((unsigned long long)s.z << 32) | s.idx;
     }
 };
@@ -265,7 +276,7 @@ __device__ __forceinline__ uint64_t scan_tiles(const ListArgs &a, uint32_t n_til
         #pragma unroll
         for (int k = 0; k < kPer; k++) {
             const uint32_t t = t0 + threadIdx.x * kPer + k;
-            x[k] = t < n_tiles ? a.ranges[t].y : 0u;
+            x[k] = t < n_tiles ? __ldcg(&a.ranges[t].y) : 0u;  // (counted by blocks on other SMs)
         }
     };
     load(0, c);
@@ -312,68 +323,224 @@ __device__ __forceinline__ uint64_t scan_tiles(const ListArgs &a, uint32_t n_til
     return carry;
 }
 
-// One block, only when the pairs exceed the capacity: the (depth, record id)
-// up to which the nearest records' pairs fit, by a radix selection over all
-// drawn records weighted by their pairs (11 bits a pass), then the counts of
-// the pairs that stay.  Rare and slow (one block reads all records).
-__device__ __noinline__ void cut_to_capacity(const ListArgs &a, const ViewTable &vt, uint32_t n_tiles)
+// When the pairs exceed the capacity, the nearest records' pairs stay: the (depth,
+// record id) up to which they fit is found by a radix selection over all drawn
+// records, weighted by their pairs.  Steps 0 to 2 add up the pairs by 11, 11 and
+// 10 bits of the depth, step 3 those of the last depth by record id; after each,
+// one block picks the bin in which the room ends.  Step 4 counts the tiles' pairs
+// that stay.  Maps of few records do it in the scan kernel, a cluster of
+// kCutCluster blocks; more take a launch a step, which return at once when nothing
+// is cut (see kCutInScan).  Bound by the latency of the records' loads, with few
+// warps in flight in the cluster and by the reads of all depths beyond.  Whole calls
+// that cut a quarter of their pairs, this against one block that did it all and
+// against the radix path:
+//   100k records, 113k pairs            110, 855, 144 us
+//   300k, 333k                          192, 2,306, 152 us
+//   1M, 1.2M                            403, 7,553, 185 us
+//   8M (1M in 8 views), 9.2M            641, 72,108, 531 us
+constexpr int kCutBins = 2048;
+constexpr int kCutSteps = 5;
+
+__device__ __forceinline__ int cut_shift(int step) { return step == 0 ? 21 : step == 1 ? 10 : 0; }
+
+// Bits of a record id below its bin in step 3.
+__device__ __forceinline__ int cut_id_shift(uint32_t total)
 {
-    constexpr int kBits = 11, kBins = 1 << kBits;
-    __shared__ unsigned long long hist[kBins];
-    __shared__ unsigned long long s_prefix, s_room;
-    if (threadIdx.x == 0) {
-        s_prefix = 0;
-        s_room = a.cap;
-    }
-    for (int shift = 55; shift >= 0; shift -= kBits) {  // 64 bits: digits at 55 (9 bits), 44, 33, 22, 11, 0
-        for (int k = threadIdx.x; k < kBins; k += kScanThreads) hist[k] = 0;
-        __syncthreads();
-        const unsigned long long prefix = s_prefix;
-        #pragma unroll 4
-        for (uint64_t r = threadIdx.x; r < a.total; r += kScanThreads) {
-            const uint32_t c = a.tt[r];
-            if (!c) continue;
-            const unsigned long long key =
-                ((unsigned long long)__float_as_uint(a.rec[12 * r + 2]) << 32) | (unsigned long long)r;
-            if (shift == 55 || (key >> (shift + kBits)) == (prefix >> (shift + kBits)))
-                atomicAdd(&hist[(key >> shift) & (kBins - 1)], (unsigned long long)c);
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long room = s_room;
-            int d = 0;
-            while (d < kBins - 1 && hist[d] <= room) room -= hist[d++];
-            s_room = room;
-            s_prefix = prefix | ((unsigned long long)d << shift);
-        }
-        __syncthreads();
-    }
-    const ListState cut = {0u, 1u, (uint32_t)(s_prefix >> 32), (uint32_t)s_prefix, (uint32_t)s_room};
-    if (threadIdx.x == 0) *a.state = cut;
-    for (uint32_t t = threadIdx.x; t < n_tiles; t += kScanThreads) a.ranges[t] = make_uint2(0u, 0u);
-    __threadfence();
-    __syncthreads();
-    for (int v = 0; v < vt.n_views; v++)
-        walk_view<true>(a, vt.v[v], v, threadIdx.x / 32, kScanThreads / 32,
-                        CutPut{cut, a.ranges + vt.v[v].tile_base, nullptr});
-    __threadfence();
-    __syncthreads();
+    const int bits = 32 - __clz((int)(total - 1));
+    return bits > 11 ? bits - 11 : 0;
 }
 
+// This thread's share (records first, first + stride, ...) of a step's sums, into
+// hist in shared memory.  z: the bits of the depth that are known.
+__device__ __forceinline__ void cut_sums(const ListArgs &a, int step, uint32_t z, unsigned long long *hist,
+                                         uint64_t first, uint64_t stride)
+{
+    constexpr int kAhead = 8;
+    const int known = step == 0 ? 32 : step == 1 ? 21 : step == 2 ? 10 : 0;  // the bits above are known
+    const int shift = cut_shift(step), id_shift = cut_id_shift(a.total);
+    for (uint64_t r0 = first; r0 < a.total; r0 += kAhead * stride) {
+        uint32_t c[kAhead], d[kAhead];
+        #pragma unroll
+        for (int k = 0; k < kAhead; k++) {
+            const uint64_t r = r0 + k * stride;
+            c[k] = r < a.total ? a.tt[r] : 0u;
+        }
+        #pragma unroll
+        for (int k = 0; k < kAhead; k++) d[k] = c[k] ? __float_as_uint(a.rec[12 * (r0 + k * stride) + 2]) : 0u;
+        #pragma unroll
+        for (int k = 0; k < kAhead; k++) {
+            if (!c[k] || (known < 32 && ((d[k] ^ z) >> known) != 0)) continue;
+            const uint32_t bin = step == 3 ? (uint32_t)(r0 + k * stride) >> id_shift : (d[k] >> shift) & (kCutBins - 1);
+            // lanes with the same bin (nearly all of them in step 0) add once
+            const uint32_t same = __match_any_sync(__activemask(), bin);
+            const uint32_t sum = __reduce_add_sync(same, c[k]);
+            if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(hist + bin, (unsigned long long)sum);
+        }
+    }
+}
+
+// Sum of the block's kScanThreads values in front of this thread's, and of all.
+__device__ __forceinline__ uint64_t scan_before(uint64_t x, uint64_t *tmp, uint64_t *total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint64_t inc = x;
+    #pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(kFullMask, inc, o);
+        if (lane >= o) inc += y;
+    }
+    __syncthreads();  // tmp is free
+    if (lane == 31) tmp[warp] = inc;
+    __syncthreads();
+    const uint64_t w = tmp[lane];
+    uint64_t wi = w;
+    #pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(kFullMask, wi, o);
+        if (lane >= o) wi += y;
+    }
+    *total = __shfl_sync(kFullMask, wi, 31);
+    return __shfl_sync(kFullMask, wi - w, warp) + inc - x;
+}
+
+// One block: the bin in which the room ends, from the sums of bins 2 tid and
+// 2 tid + 1, into the state; after step 3 the record, among those of the bin.
+__device__ __forceinline__ void cut_pick(const ListArgs &a, int step, unsigned long long h0, unsigned long long h1)
+{
+    __shared__ uint64_t tmp[32];
+    __shared__ uint32_t s_bin, s_found;
+    const uint64_t room = __ldcg(&a.state->room);
+    const uint32_t z = __ldcg(&a.state->cut_z);
+    uint64_t all;
+    const uint64_t before = scan_before(h0 + h1, tmp, &all);
+    if (threadIdx.x == 0) s_bin = 0;
+    __syncthreads();  // every thread has read the state
+    if (before <= room && room < before + h0 + h1) {  // one thread's: the sums exceed the room
+        const bool second = room >= before + h0;
+        const uint32_t bin = 2 * threadIdx.x + second;
+        s_bin = bin;
+        if (step < 3) a.state->cut_z = z | (bin << cut_shift(step));
+        a.state->room = room - before - (second ? h0 : 0);
+    }
+    if (threadIdx.x == 0) s_found = 0;
+    __threadfence();
+    __syncthreads();
+    if (step < 3) return;
+    const int id_shift = cut_id_shift(a.total);
+    uint64_t left = __ldcg(&a.state->room);
+    const uint64_t r0 = (uint64_t)s_bin << id_shift, r1 = r0 + (1ull << id_shift);
+    for (uint64_t b = r0; b < r1; b += kScanThreads) {
+        const uint64_t r = b + threadIdx.x;
+        uint32_t c = r < r1 && r < a.total ? a.tt[r] : 0u;
+        if (c && __float_as_uint(a.rec[12 * r + 2]) != z) c = 0;
+        const uint64_t at = scan_before(c, tmp, &all);
+        if (at <= left && left < at + c) {
+            a.state->cut_r = (uint32_t)r;
+            a.state->cut_pairs = (uint32_t)(left - at);
+            s_found = 1;
+        }
+        __threadfence();
+        __syncthreads();
+        if (s_found) break;
+        left -= all;
+    }
+}
+
+// Step 4, the warps from `first` on of `stride`: the pairs that stay, in the
+// ranges' ends (cleared before).
+__device__ __forceinline__ void cut_count(const ListArgs &a, const ViewTable &vt, uint32_t first, uint32_t stride)
+{
+    ListState cut = {};
+    cut.cut_z = __ldcg(&a.state->cut_z);
+    cut.cut_r = __ldcg(&a.state->cut_r);
+    cut.cut_pairs = __ldcg(&a.state->cut_pairs);
+    for (int v = 0; v < vt.n_views; v++)
+        walk_view<true>(a, vt.v[v], v, first, stride, CutPut{cut, a.ranges + vt.v[v].tile_base, nullptr});
+}
+
+// CLUSTER: a cluster of kCutCluster blocks, of which the first scans and all cut
+// when the pairs do not fit.  Otherwise one block, which leaves a cut to the
+// launches behind it.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kScanThreads) tile_scan_kernel(ListArgs a, ViewTable vt, bool advance)
 {
     chain_go();
     chain_wait();
-    const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
-    if (threadIdx.x == 0) *a.state = ListState{};
-    const uint64_t pairs = scan_tiles(a, n_tiles, advance);
-    if (threadIdx.x == 0) {
-        *a.n_pairs = pairs > 0xffffffffull ? 0xffffffffu : (uint32_t)pairs;
-        if (pairs > a.cap) raise_status(a.status, GS_ERR_CAPACITY);
+    const uint32_t n_tiles = (uint32_t)vt.n_tiles_total, rank = CLUSTER ? cluster_rank() : 0u;
+    if (rank == 0) {
+        if (threadIdx.x == 0) *a.state = ListState{};
+        const uint64_t pairs = scan_tiles(a, n_tiles, advance);
+        if (threadIdx.x == 0) {
+            *a.n_pairs = pairs > 0xffffffffull ? 0xffffffffu : (uint32_t)pairs;
+            if (pairs > a.cap) {
+                raise_status(a.status, GS_ERR_CAPACITY);
+                a.state->cut = 1;
+                a.state->room = a.cap;
+            }
+        }
+        if (!CLUSTER && pairs > a.cap)
+            for (int k = threadIdx.x; k < kCutBins; k += kScanThreads) a.cut_hist[k] = 0;
     }
-    if (pairs > a.cap) {  // block-uniform
+    if constexpr (CLUSTER) {
+        __shared__ unsigned long long hist[kCutBins];
+        cluster_sync();
+        if (!__ldcg(&a.state->cut)) return;
+        const uint32_t first = rank * kScanThreads + threadIdx.x, stride = kCutCluster * kScanThreads;
+        for (uint32_t t = first; t < n_tiles; t += stride) a.ranges[t] = make_uint2(0u, 0u);
+        for (int step = 0; step < kCutSteps - 1; step++) {
+            for (int k = threadIdx.x; k < kCutBins; k += kScanThreads) hist[k] = 0;
+            __syncthreads();
+            cut_sums(a, step, __ldcg(&a.state->cut_z), hist, first, stride);
+            cluster_sync();  // every block's sums are complete
+            if (rank == 0) {
+                unsigned long long h[2] = {};
+                for (int b = 0; b < kCutCluster; b++)
+                    for (int k = 0; k < 2; k++) h[k] += ld_cluster(hist + 2 * threadIdx.x + k, b);
+                cut_pick(a, step, h[0], h[1]);
+            }
+            cluster_sync();  // the state is written, the sums are read
+        }
+        cut_count(a, vt, first / 32, stride / 32);
+        cluster_sync();
+        if (rank == 0) scan_tiles(a, n_tiles, true);
+    }
+}
+
+// A step of the cut over the whole GPU; the last block to end picks the bin or
+// scans the tiles.
+__global__ void __launch_bounds__(kScanThreads) tile_cut_kernel(ListArgs a, ViewTable vt, int step)
+{
+    chain_go();
+    chain_wait();
+    if (!a.state->cut) return;
+    __shared__ unsigned long long hist[kCutBins];
+    __shared__ bool s_last;
+    const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
+    const uint32_t first = blockIdx.x * kScanThreads + threadIdx.x, stride = gridDim.x * kScanThreads;
+    if (step < kCutSteps - 1) {
+        if (step == 0)
+            for (uint32_t t = first; t < n_tiles; t += stride) a.ranges[t] = make_uint2(0u, 0u);
+        for (int k = threadIdx.x; k < kCutBins; k += kScanThreads) hist[k] = 0;
         __syncthreads();
-        cut_to_capacity(a, vt, n_tiles);
+        cut_sums(a, step, a.state->cut_z, hist, first, stride);
+        __syncthreads();
+        for (int k = threadIdx.x; k < kCutBins; k += kScanThreads)
+            if (hist[k]) atomicAdd(a.cut_hist + k, hist[k]);
+    } else {
+        cut_count(a, vt, first / 32, stride / 32);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&a.state->arrived, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) a.state->arrived = 0;
+    if (step < kCutSteps - 1) {
+        const unsigned long long h0 = __ldcg(a.cut_hist + 2 * threadIdx.x), h1 = __ldcg(a.cut_hist + 2 * threadIdx.x + 1);
+        a.cut_hist[2 * threadIdx.x] = a.cut_hist[2 * threadIdx.x + 1] = 0;
+        cut_pick(a, step, h0, h1);
+    } else {
         scan_tiles(a, n_tiles, true);
     }
 }
@@ -834,7 +1001,13 @@ static gs_status_t launch_walks(const ListArgs &a, const ViewTable &vt, uint32_t
         return GS_ERR_CUDA;
     gs_status_t st = launch_chained(tile_count_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
     if (st != GS_OK) return st;
-    st = launch_chained(tile_scan_kernel, 1, kScanThreads, 0, s, a, vt, !PRIVATE);
+    if (a.total <= kCutInScan) {
+        st = launch_with(true, kCutCluster, tile_scan_kernel<true>, kCutCluster, kScanThreads, 0, s, a, vt, !PRIVATE);
+    } else {
+        st = launch_chained(tile_scan_kernel<false>, 1, kScanThreads, 0, s, a, vt, !PRIVATE);
+        for (int step = 0; step < kCutSteps && st == GS_OK; step++)
+            st = launch_chained(tile_cut_kernel, (unsigned)num_sms(), kScanThreads, 0, s, a, vt, step);
+    }
     if (st != GS_OK) return st;
     return launch_chained(tile_scatter_kernel<PRIVATE>, grid, kListThreads, smem, s, a, vt, blocks_per_view);
 }
@@ -871,6 +1044,8 @@ gs_status_t tile_lists(const gs_projected_t *proj, int64_t total, int64_t n, con
     a.words = static_cast<unsigned long long *>(buf.words);
     a.keys = bins->keys;
     a.vals = bins->vals;
+    a.cut_hist = static_cast<unsigned long long *>(buf.table);
+    static_assert((size_t)kCutInScan * 4 >= kCutBins * sizeof(unsigned long long), "the table has room for the sums");
     const uint32_t n_tiles = (uint32_t)vt.n_tiles_total;
     gs_status_t st = launch_clear(reinterpret_cast<uint32_t *>(a.ranges), 2 * n_tiles, s);
     if (st != GS_OK) return st;

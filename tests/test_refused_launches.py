@@ -72,6 +72,7 @@ def _lookback(lib):
 CALLS = {
     "bins-private-counts": (_bin_sort(_views((1200, 680)), 300_000), 6),
     "bins-global-counts": (_bin_sort(_views((1280, 720), tile=(8, 8)), 20_000), 6),
+    "bins-cut-launches": (_bin_sort(_views((1200, 680)), 2_000_000), 11),
     "bins-radix": (_bin_sort(_views((64, 48)), 100_000), 14),
     "render-fwd": (lambda lib: lib.gs_render_fwd(ref(PROJ), 1000, ref(BINS), FULL, len(FULL), ref(IMG), AT, None), 2),
     "render-bwd-0": (_render_bwd(FULL, 0), 4),
