@@ -54,6 +54,18 @@ class FlatParams:
         return out
 
 
+def bin_kernels(n, n_views, n_tiles):
+    """Kernels launched by gs_bin_sort (clears excluded)."""
+    records = n * n_views
+    if records <= 2048 * n_tiles and n_tiles <= 1 << 18:
+        # tile count, scan, scatter, sort; the merge of long lists; the cut to the capacity of large maps
+        return 4 + (n > 8192) + 5 * (records > 1 << 20)
+    # record count, scan, compaction, 4 depth passes, pair count, scan, emission, the tile-id
+    # passes (8 bits each) and the ranges
+    tile_passes = max(1, (max(n_tiles - 1, 0).bit_length() + 7) // 8)
+    return 3 + 4 + 3 + tile_passes + 1
+
+
 class MappingStep:
     """Buffers and launches of one joint mapping / tracking iteration."""
 
@@ -206,14 +218,7 @@ class MappingStep:
 
     def kernels_per_step(self):
         """Kernels of this library launched by one run() (clears excluded)."""
-        r = self.rast
-        if r.n * r.V <= 2048 * r.n_tiles and r.n_tiles <= 1 << 18:
-            k_bin = 4 + (r.n > 8192)  # tile count, scan, scatter, sort; the merge of long lists
-        else:
-            # record count, scan, compaction, 4 depth passes, pair count, scan, emission, the tile-id
-            # passes (8 bits each) and the ranges
-            tile_passes = max(1, (max(r.n_tiles - 1, 0).bit_length() + 7) // 8)
-            k_bin = 3 + 4 + 3 + tile_passes + 1
+        k_bin = bin_kernels(self.rast.n, self.rast.V, self.rast.n_tiles)
         # project, bin, fwd (with the L1 loss), bwd, pbwd colour + geometry
         k = 1 + k_bin + 1 + 1 + 2
         k += 2 if self.zeta > 0 else 0
