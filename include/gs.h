@@ -292,15 +292,17 @@ gs_status_t gs_render_stats(const gs_projected_t *proj, int64_t n, const gs_bins
  * the list entries in shared memory: 32 loaded by the lanes into registers,
  * 32 copied by the lanes' asynchronous copies into a second buffer, or 32 or
  * 64 gathered by the tensor memory accelerator (a band that does not divide
- * a view's tile falls back to the (2, 8) band of the same staging; defaults:
- * forward 7, backward 9, the asynchronous-copy (2, 8) and (4, 8)).  All
- * variants compute the same result; the autotuner times them on the workload
- * and sets the fastest.  Until they are set, images of few pixels take the
- * (1, 8) and (2, 8) bands of the default staging.  The setting is process-wide and read when a kernel
- * is launched.  GS_ERR_INVALID_ARG for an index out of range. */
+ * a view's tile falls back to the (2, 8) band of the same staging).  -1, for
+ * either, is the library's own choice and the state at the start: forward 7,
+ * backward 9, the asynchronous-copy (2, 8) and (4, 8), and for images of few
+ * pixels the (1, 8) and (2, 8) bands of the same staging.  All variants compute
+ * the same result; the autotuner times them on the workload and sets the
+ * fastest.  The setting is process-wide and read when a kernel is launched.
+ * GS_ERR_INVALID_ARG for an index out of range. */
 gs_status_t gs_set_render_variants(int32_t fwd, int32_t bwd);
 
-/* Current variants and the number of each (any pointer may be NULL). */
+/* Current variants (-1: the library's own choice) and the number of each (any
+ * pointer may be NULL).  Setting what was got restores the state. */
 gs_status_t gs_get_render_variants(int32_t *fwd, int32_t *bwd, int32_t *n_fwd, int32_t *n_bwd);
 
 /* a6. L1 rendering losses with the optional filter gate (Sec. 3.3

@@ -184,11 +184,12 @@ def gs_render_stats(proj, n, bins, views, n_eval, n_blend, work_counter, stream=
 
 
 def gs_set_render_variants(fwd, bwd):
+    """Pins the compositing variants for the process; -1 leaves one to the library."""
     check(lib().gs_set_render_variants(int(fwd), int(bwd)), "gs_set_render_variants")
 
 
 def gs_get_render_variants():
-    """(fwd, bwd, n_fwd, n_bwd): variants in use and how many exist."""
+    """(fwd, bwd, n_fwd, n_bwd): variants set (-1: the library's choice) and how many exist."""
     out = [ctypes.c_int32() for _ in range(4)]
     check(lib().gs_get_render_variants(*[ctypes.byref(o) for o in out]), "gs_get_render_variants")
     return tuple(o.value for o in out)

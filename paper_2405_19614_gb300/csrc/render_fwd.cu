@@ -628,14 +628,15 @@ extern "C" gs_status_t gs_render_stats(const gs_projected_t *proj, int64_t n, co
     return launch_fwd<1, 16, 32, false, true>(a, vt, none, s);
 }
 
-// Compositing kernel variants in use (see kFwdVariants), set by the
-// autotuner; defaults suit 1200x680 views of room-scale scenes.
+// Compositing kernel variants in use (see kFwdVariants), set by the autotuner;
+// -1, the start: by pixel count, below.
 namespace gs {
-static int g_variant_fwd = 7;  // (2, 8) bands, asynchronous-copy staging
-static int g_variant_bwd = 9;  // (4, 8) bands, asynchronous-copy staging
-static bool g_variants_set = false;
+static int g_variant_fwd = -1;
+static int g_variant_bwd = -1;
 
-// Until variants are set, few pixels take smaller bands: where a launch has
+// Without a set variant, views of room-scale scenes take 7 and 9, the
+// asynchronous-copy (2, 8) and (4, 8) bands (right for 1200x680), and few pixels
+// smaller bands of the same staging: where a launch has
 // fewer bands than the GPU holds warps, the longest list of one band is the
 // launch's time, and a band of fewer pixels walks its list faster.  The lines
 // are where both sides measured alike; with `held` warps of a 4-warp, 8-block
@@ -649,24 +650,24 @@ static bool g_variants_set = false;
 //     50 on 254k.
 int render_variant_fwd(int64_t n_pix)
 {
+    const int set = g_variant_fwd;
     const int64_t held = (int64_t)num_sms() * 32;
-    return !g_variants_set && n_pix / 32 <= held / 2 ? 6 : g_variant_fwd;
+    return set >= 0 ? set : n_pix / 32 <= held / 2 ? 6 : 7;
 }
 
 int render_variant_bwd(int64_t n_pix)
 {
+    const int set = g_variant_bwd;
     const int64_t held = (int64_t)num_sms() * 32;
-    if (g_variants_set) return g_variant_bwd;
-    return n_pix / 32 <= held / 2 ? 6 : n_pix / 64 <= held * 13 / 20 ? 7 : g_variant_bwd;
+    return set >= 0 ? set : n_pix / 32 <= held / 2 ? 6 : n_pix / 64 <= held * 13 / 20 ? 7 : 9;
 }
 }  // namespace gs
 
 extern "C" gs_status_t gs_set_render_variants(int32_t fwd, int32_t bwd)
 {
-    if (fwd < 0 || fwd >= kFwdVariants || bwd < 0 || bwd >= kBwdVariants) return GS_ERR_INVALID_ARG;
+    if (fwd < -1 || fwd >= kFwdVariants || bwd < -1 || bwd >= kBwdVariants) return GS_ERR_INVALID_ARG;
     g_variant_fwd = fwd;
     g_variant_bwd = bwd;
-    g_variants_set = true;
     return GS_OK;
 }
 
