@@ -607,6 +607,24 @@ def oracle_view_sample(c, v, rows=None):
                       f"Gaussians projected) in one thread, {sec:.1f} s"}
 
 
+def tuned_summary(tuned):
+    """What the JSON line says of the autotuner: the shape and variants picked
+    and each tile shape's time, without those of every variant on every shape
+    (4 KB a workload)."""
+    if not tuned or "candidates" not in tuned:
+        return tuned
+    return dict(tuned, candidates={tile: c["total_ms"] for tile, c in tuned["candidates"].items()})
+
+
+def printed(x):
+    """x with its floats to seven digits: a line that the last 8 KB of a log hold."""
+    if isinstance(x, dict):
+        return {k: printed(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [printed(v) for v in x]
+    return float(f"{x:.7g}") if isinstance(x, float) else x
+
+
 def measure_mapping_config(idx, args, device, with_plain):
     """A mapping workload measured like the headline: autotuned variants, the
     step replayed as a CUDA graph, per-stage events in an eager pass, the
@@ -654,7 +672,7 @@ def measure_mapping_config(idx, args, device, with_plain):
            "stages": {k: round(v, 4) for k, v in stage_ms.items()},
            "roofline": dict(stage_roofline(dom, stage_ms, works, hbm_peak, alu_peak), kernel=dom),
            "roofline_step": {"floor_ms": floor, "ms": ms, "frac": floor / ms},
-           "tuned": tuned}
+           "tuned": tuned_summary(tuned)}
     if with_plain and step.rast.V > 1:
         rs = plain_steps(c, step, cap, device)
         for _ in range(2):
@@ -1163,7 +1181,7 @@ def main_ours(args):
         "e2e": {"value": world * px_per_step / e2e_ms / 1e3, "unit": "Mpix/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": 4},
         "gpu_launches": launches,
-        "tuned": tuned,
+        "tuned": tuned_summary(tuned),
         "stages": stages,
         "work": w,
         "roofline": roofline,
@@ -1180,7 +1198,7 @@ def main_ours(args):
         "configs": configs,
     }
     if rank == 0:
-        print(json.dumps(out))
+        print(json.dumps(printed(out)))
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
