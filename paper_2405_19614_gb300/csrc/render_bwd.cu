@@ -57,7 +57,7 @@ struct RenderBwdArgs {
     const uint32_t *n_contrib;
     const float *d_rgb, *d_depth, *d_alpha;
     float *grad2d;
-    uint32_t *work_counter;  // null: the warps take the items in order, one each
+    uint32_t *work_counter;
     uint32_t *status;  // device error word (a bounded wait that expired), may be null
     uint32_t n_items;  // (view, tile, band) work items, set by the launcher
 };
@@ -108,7 +108,10 @@ __device__ __forceinline__ void load_bwd_entry(const RenderBwdArgs &a, int64_t r
 // second shared-memory buffer with their own asynchronous copies (through L1,
 // like the lane loads, but holding no registers), and load the Gaussian
 // indices one chunk further ahead.
-template <int PPT, int BW, int CH, bool TMA, bool ASYNC = false>
+// COUNTED: warps draw their items from the work counter; else (small images)
+// warp w of the grid has item w alone.  (A branch on the counter's pointer in one
+// kernel cost the walk 2.4 %: 1.461 against 1.427 ms on the 1M-Gaussian step.)
+template <int PPT, int BW, int CH, bool TMA, bool ASYNC, bool COUNTED>
 __global__ void __launch_bounds__(kRenderThreads, RenderOccupancy<PPT, TMA || ASYNC>::bwd)
     render_bwd_kernel(RenderBwdArgs a, ViewTable vt, const __grid_constant__ CUtensorMap rec_map)
 {
@@ -153,10 +156,10 @@ __global__ void __launch_bounds__(kRenderThreads, RenderOccupancy<PPT, TMA || AS
     const int red_entry = lane / kPairs, red_pair = lane % kPairs;  // the row this lane adds up
     for (uint32_t turn = 0;; turn++) {
         uint32_t wi = 0;
-        if (a.work_counter) {
+        if (COUNTED) {
             if (lane == 0) wi = atomicAdd(a.work_counter, 1u);
             wi = __shfl_sync(kFullMask, wi, 0);
-        } else {  // a warp an item: nothing to hand out
+        } else {
             wi = turn == 0 ? blockIdx.x * WARPS + warp : a.n_items;
         }
         if (wi >= a.n_items) break;
@@ -567,21 +570,18 @@ static gs_status_t launch_bwd(RenderBwdArgs a, ViewTable vt, const CUtensorMap &
 {
     // work items: the bands of every tile of every view (tile shapes are per view)
     a.n_items = render_items(&vt, BW, PPT * (32 / BW));
-    auto kern = render_bwd_kernel<PPT, BW, CH, TMA, ASYNC>;
+    auto kern = render_bwd_kernel<PPT, BW, CH, TMA, ASYNC, true>;
     static PerDevice per_sm;
     const int64_t slots = (int64_t)num_sms() * blocks_per_sm(per_sm, kern, kRenderThreads);
     const int64_t blocks_needed = ((int64_t)a.n_items + kRenderThreads / 32 - 1) / (kRenderThreads / 32);
-    const int grid = (int)(slots < blocks_needed ? slots : blocks_needed);
-    // every item has a warp of its own when the grid holds them all: no counter
+    // every item has a warp of its own when the GPU holds them all: no counter
     // to clear and none to wait for (2 us less of a small image)
-    const bool counted = blocks_needed > slots;
-    if (counted) {
-        const gs_status_t st = launch_clear(a.work_counter, 1, s);
-        if (st != GS_OK) return st;
-    } else {
-        a.work_counter = nullptr;
-    }
-    return launch_with(counted, 1, kern, grid > 0 ? grid : 1, kRenderThreads, 0, s, a, vt, map);
+    if (blocks_needed <= slots)
+        return launch_with(false, 1, render_bwd_kernel<PPT, BW, CH, TMA, ASYNC, false>,
+                           blocks_needed > 0 ? (unsigned)blocks_needed : 1u, kRenderThreads, 0, s, a, vt, map);
+    const gs_status_t st = launch_clear(a.work_counter, 1, s);
+    if (st != GS_OK) return st;
+    return launch_with(true, 1, kern, (unsigned)slots, kRenderThreads, 0, s, a, vt, map);
 }
 
 template <int CH, bool TMA, bool ASYNC = false>

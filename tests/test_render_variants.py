@@ -54,3 +54,18 @@ def test_saved_variants_restore_the_own_choice(fake):
         assert fake.lib.gs_set_render_variants(*bad) == 1
     assert fake.lib.gs_set_render_variants(fwd, bwd) == 0
     assert {s: _bands(fake, s) for s in OWN} == OWN
+
+
+def test_the_backward_hands_out_items_where_they_outnumber_the_warps(fake):
+    """Kernels of their own with and without the work counter (a branch inside one
+    slowed the long walks by 2.4 %)."""
+    def kernels(size, count):
+        views = gs.make_views([[300.0, 300.0, size[0] / 2, size[1] / 2]] * count, [size] * count)
+        proj, bins, img = GsProjected(*[AT] * 5), GsBins(*[AT] * 5, 1 << 20), GsImage(*[AT] * 5)
+        status, _, events = fake.run(lambda lib: lib.gs_render_bwd_splats(
+            ref(proj), 1000, ref(bins), views, count, ref(img), AT, AT, None, AT, AT, None))
+        assert status == 0
+        return [name for what, name, _ in events if what == "launch"]
+    small, large = kernels((64, 48), 1), kernels((1200, 680), 8)
+    assert len(small) == 1 and "render_bwd_kernelILi1ELi8ELi32ELb0ELb1ELb0EE" in small[0]
+    assert len(large) == 2 and "render_bwd_kernelILi4ELi8ELi32ELb0ELb1ELb1EE" in large[1]
