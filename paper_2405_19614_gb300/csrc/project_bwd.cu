@@ -24,9 +24,9 @@
 //
 // Bound by latency and, where many views draw a Gaussian, instruction issue.
 // Warps walk only the views that draw one of their Gaussians, and only those
-// store and sum twist terms: colour 113 -> 97 us and geometry 77 -> 68 us for 1M
-// Gaussians in 8 views, 679 -> 640 and 598 -> 523 us for 4M in 16 (most Gaussians
-// of a floor are drawn in few of its views).
+// store and sum twist terms: colour 114 -> 96 us and geometry 77 -> 68 us for 1M
+// Gaussians in 8 views, 685 -> 649 and 603 -> 528 us for 4M in 16 (most Gaussians
+// of a floor are drawn in few of its views; all under ncu).
 #include "chain.cuh"
 #include "common.cuh"
 #include "async_copy.cuh"
