@@ -463,7 +463,8 @@ extern "C" gs_status_t gs_bin_sort(const gs_projected_t *proj, int64_t n, const 
     const int tile_passes = (bits_for(vt.n_tiles_total - 1) + 7) / 8 > 0 ? (bits_for(vt.n_tiles_total - 1) + 7) / 8 : 1;
     if (tile_passes > kMaxTilePasses) return GS_ERR_INVALID_ARG;
     cudaStream_t s = as_stream(stream);
-    if (total > 0 && tile_lists_fit(total, vt.n_tiles_total)) {
+    // (the tile lists read and write the ranges as pairs of words)
+    if (total > 0 && tile_lists_fit(total, vt.n_tiles_total) && !(reinterpret_cast<uintptr_t>(bins->ranges) & 7)) {
         if (!proj->rec || !proj->rect || !proj->tiles_touched || !proj->tile_mask) return GS_ERR_INVALID_ARG;
         // the pair buffer holds the 64-bit words, a look-back region the list of
         // long tiles' chunks, the record buffers (rz to recs, one after the
