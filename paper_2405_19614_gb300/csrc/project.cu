@@ -131,7 +131,8 @@ __device__ __forceinline__ bool world_covariance(const float ls[3], const float 
 // 3 (sqrt(|S|) sqrt(|W W^T| F) / |z| + sqrt(blur)) + 1.  The bound is taken a
 // thousandth and a pixel larger, far above the rounding of both sides, and the
 // mean from an approximate reciprocal within 1e-5 of its terms; whatever is not
-// finite fails the comparisons and goes on to the contract.  reach: the view's
+// finite fails the comparisons and goes on to the contract, as does a depth
+// beyond the fast quotient's range (above 2^126 it gives zero).  reach: the view's
 // 3.003 sqrt(|W W^T| F) and 3.003 sqrt(blur) + 2.  (4M Gaussians, 16 views:
 // 766 -> 725 us for the kernel; 1M, 8 views: 100 -> 90.)
 __device__ __forceinline__ bool beside_the_image(float x, float y, float z, float root_s, const float *reach,
@@ -142,8 +143,8 @@ __device__ __forceinline__ bool beside_the_image(float x, float y, float z, floa
     const float px = V.fx * x * rz, py = V.fy * y * rz;
     const float ru = fmaf(1e-5f, fabsf(px) + fabsf(V.cx), r), rv = fmaf(1e-5f, fabsf(py) + fabsf(V.cy), r);
     const float u = px + V.cx, v = py + V.cy;
-    return u + ru < 0.0f || v + rv < 0.0f || u - ru > (float)(V.tiles_x * V.tile_w) ||
-           v - rv > (float)(V.tiles_y * V.tile_h);
+    return fabsf(z) < 0x1p126f && (u + ru < 0.0f || v + rv < 0.0f || u - ru > (float)(V.tiles_x * V.tile_w) ||
+                                   v - rv > (float)(V.tiles_y * V.tile_h));
 }
 
 // Largest absolute row sum (the infinity norm) of a 3 x 3 matrix.
