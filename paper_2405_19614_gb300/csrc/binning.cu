@@ -4,7 +4,7 @@
 //
 // The result is the list a stable sort of the 64-bit keys (global tile << 32)
 // | bits(depth), values = Gaussian index, would give: per tile, entries by
-// depth, equal depths in index order.  Unless the map crowds few tiles,
+// depth, equal depths in index order.  Up to 2,048 records a tile on average
 // tile_lists.cu builds it tile by tile; here it is built in two small sorts
 // instead of one wide one:
 //   1. the drawn (view, Gaussian) records are compacted and sorted by depth
