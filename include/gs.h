@@ -221,8 +221,10 @@ size_t gs_bin_sort_workspace_size(int64_t n_records, int64_t pair_capacity, int6
  * equal depths in index order, and each tile's [start, end) ([0, 0) when
  * empty).  Built by counting each tile's pairs, scattering them to their tiles
  * and sorting each tile's list, or, above 2,048 records a tile on average and
- * for ranges that are not 8-byte aligned (a slower path), by sorting the drawn records by depth, emitting their pairs in that order and sorting the
- * pairs stably by tile id (onesweep radix passes over 32-bit keys).  n_views * n must be below 2^32.  When the pair
+ * for ranges that are not 8-byte aligned (a slower path), by sorting the drawn
+ * records by depth, emitting their pairs in that order and sorting the pairs
+ * stably by tile id (onesweep radix passes over 32-bit keys).  n_views * n must
+ * be below 2^32.  When the pair
  * total exceeds bins->capacity, n_pairs still reports the total, the
  * capacity bit is set in the status word and only the pairs of the nearest
  * records that fit are binned.
